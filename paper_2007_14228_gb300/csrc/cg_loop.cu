@@ -1,0 +1,451 @@
+// The Hartree CG with the separable preconditioner as one persistent cooperative kernel.
+//
+// A CG iteration is five dependent phases (lattice SpMV; update and forward pass; middle pass;
+// backward pass; direction), each a few microseconds of work below half a million nodes.  As
+// kernels of their own (ten launches with the six-pass preconditioner) they cost 112 us per
+// iteration at 49^3 nodes, most of it launch latency, reloading the axis matrices and draining;
+// here one CTA per SM keeps the six axis matrices, the stencil tables and its tensor memory for
+// the whole solve, the phases are separated by grid barriers, and the residual test (with the
+// iteration counts it is taken at) runs on the device, so a solve is one launch and one host
+// synchronization: 44 us per iteration at 49^3 nodes (float64 SpMV 10, forward 6, middle 4,
+// backward 6, direction 3, five barriers at 1.5 and the two scalars at 2), 92 against 190 at
+// 121x65x61 (float-float SpMV 31).  float64 operations of a warp take 16 cycles each, so the
+// passes that run on few SMs hold as few of them as possible.  512 threads and eight loads in
+// flight per lane measured best (256: 50 us at 49^3 and 120 at 121x65x61; 768: 49 and 102).
+//
+// Sums over the grid go through one partial per CTA, written before a barrier and added in CTA
+// order by every CTA after it.  A barrier wait is bounded: on timeout the CTA raises the abort
+// flag, which every other wait polls, and the host returns OFKS_ETIMEOUT.
+#include <algorithm>
+#include <cmath>
+
+#include "sep_plane.cuh"
+
+namespace {
+
+using namespace sepp;
+
+constexpr int NTH = 512, NW = NTH / 32;
+constexpr int BATCH = 8;                          // stencil entries whose loads are issued together
+constexpr int SPLIT_ROW = 40;                     // rows of more entries are shared by two lanes
+constexpr long long BAR_WAIT = 1LL << 21;
+
+struct CgOut {
+    double rr, bb, rate;
+    int it, status, abort;
+    unsigned bar;
+};
+
+struct Loop {
+    int nx, ny, nz, px, py, pz, ncol, NT;
+    const bf *S[3], *St[3];
+    const float *lx, *lyzp;
+    float *T;
+    uint32_t oSt[3], oS[3], oB, part_p, part_m;   // shared-memory offsets; bytes per data part
+    int tcols;
+    Vecs V;
+    double *p;
+    float *zf;                                    // z, float32 (in the room of the float64 z)
+    float2 *pf;                                   // p as float32 pairs (float-float SpMV); null: float64
+    const double *rhs;
+    double *q;
+    int Lx;
+    const StencilType *types;
+    const StencilCode *code;
+    const double *val;
+    const float2 *valff;
+    double tol2, rate;
+    int max_iter;
+    double *part;                                 // 4 x gridDim.x: pq, rr, rz, |rhs|^2
+    CgOut *out;
+};
+
+// barrier over the grid; target counts this CTA's arrivals times the grid.  False after an abort.
+__device__ __forceinline__ bool grid_barrier(CgOut *out, unsigned &target, int *s_abort) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        target += gridDim.x;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&out->bar) : "memory");
+        bool ok = false;
+        for (long long w = 0; w < BAR_WAIT; ++w) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&out->bar) : "memory");
+            if ((int)(v - target) >= 0) { ok = true; break; }
+            if ((w & 63) == 63 && *(volatile int *)&out->abort) break;
+        }
+        if (!ok) { atomicExch(&out->abort, 1); *s_abort = 1; }
+    }
+    __syncthreads();
+    return *s_abort == 0;
+}
+
+// sum of the CTAs' partials in CTA order, by every CTA
+__device__ __forceinline__ double grid_total(const double *part, double *s_val) {
+    if (threadIdx.x < 32) {
+        double s = 0.0;
+        for (unsigned i = threadIdx.x; i < gridDim.x; i += 32) s += __ldcg(part + i);
+        s = warp_sum(s);
+        if (threadIdx.x == 0) *s_val = s;
+    }
+    __syncthreads();
+    return *s_val;
+}
+
+struct Tables {
+    StencilType type[8];
+    StencilCode code[8 * ST_MAXE];
+    int wblk[9];                                  // first block of each type (one warp's rows)
+};
+
+// a row of the stencil, or this lane's part of it: entries [e0, e1) of its type, its lattice
+// position and node, and its index in the four parity classes
+struct Row {
+    int t, e0, e1, a, b, c, node, idx[4];
+};
+
+// the row's product with x over its entries in the order of the stencil kernels, BATCH loads at a time
+template <class F2, class Get, class Acc>
+__device__ __forceinline__ void row_product(const Tables &tb, const Row &R, const F2 *__restrict__ val, Get get, Acc acc) {
+    const StencilCode *se = tb.code + R.t * ST_MAXE;
+    auto fetch = [&](const StencilCode &E, F2 &v, F2 &x) {
+        const int lo = E.lin4 & 1 ? R.idx[1] : R.idx[0], hi = E.lin4 & 1 ? R.idx[3] : R.idx[2];
+        v = __ldg(val + E.off + (E.lin4 & 2 ? hi : lo));
+        x = get(R.node + (E.lin4 >> 2));
+    };
+    F2 v[BATCH], x[BATCH];
+    int e = R.e0;
+    for (; e + BATCH <= R.e1; e += BATCH) {
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) fetch(se[e + u], v[u], x[u]);
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) acc(v[u], x[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < BATCH - 1; ++u)           // the rest, its loads together too
+        if (e + u < R.e1) fetch(se[e + u], v[u], x[u]);
+#pragma unroll
+    for (int u = 0; u < BATCH - 1; ++u)
+        if (e + u < R.e1) acc(v[u], x[u]);
+}
+
+__device__ __forceinline__ void ff_madd(float &sh, float &sl, const float2 a, const float2 x) {
+    const float p = __fmul_rn(a.x, x.x);
+    float e = __fmaf_rn(a.x, x.x, -p);
+    e = __fmaf_rn(a.x, x.y, e);
+    e = __fmaf_rn(a.y, x.x, e);
+    const float t = __fadd_rn(sh, p);
+    const float bv = __fsub_rn(t, sh);
+    const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bv)), __fsub_rn(p, bv));
+    sh = t;
+    sl = __fadd_rn(sl, __fadd_rn(err, e));
+}
+
+// Rows in blocks of one node type, 32 per warp or, where a row is long (cell vertices, 65 entries),
+// 16 with two lanes to a row, dealt to the grid's CTAs in turn and within a CTA to the warps forth and
+// back: s = product(row) over the row's interior entries, then done(row, s) on one lane per row
+// (interior or not).
+template <class Product, class Done>
+__device__ __forceinline__ void for_rows(const Loop &P, const Tables &tb, Product product, Done done) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int round = 0; round * NW * (int)gridDim.x < tb.wblk[8]; ++round) {
+        const int k = round * NW + (round & 1 ? NW - 1 - warp : warp);
+        const int wb = k * (int)gridDim.x + (int)blockIdx.x;
+        if (wb >= tb.wblk[8]) continue;           // the same for the whole warp
+        int t = 0;
+        while (wb >= tb.wblk[t + 1]) ++t;
+        const StencilType &T = tb.type[t];
+        const bool two = T.nent > SPLIT_ROW;
+        const int idx = two ? (wb - tb.wblk[t]) * 16 + (lane & 15) : (wb - tb.wblk[t]) * 32 + lane;
+        const int nyz = T.ny * T.nz, ia = idx / nyz, rem = idx - ia * nyz, ib = rem / T.nz, ic = rem - ib * T.nz;
+        Row R;
+        R.t = t; R.a = 2 * ia + T.px; R.b = 2 * ib + T.py; R.c = 2 * ic + T.pz;
+        R.node = (R.a * P.V.Ly + R.b) * P.V.Lz + R.c;
+        const int half = (T.nent + 1) >> 1;
+        R.e0 = two && lane >= 16 ? half : 0;
+        R.e1 = two && lane < 16 ? half : T.nent;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {             // class q: extents of the sub-lattices of that parity
+            const int ny = (P.V.Ly - (q >> 1) + 1) >> 1, nz = (P.V.Lz - (q & 1) + 1) >> 1;
+            R.idx[q] = (ia * ny + ib) * nz + ic;
+        }
+        const bool in = idx < T.n && R.a > 0 && R.a < P.Lx - 1 && R.b > 0 && R.b < P.V.Ly - 1 && R.c > 0 && R.c < P.V.Lz - 1;
+        double s = in ? product(R) : 0.0;
+        if (two) s += __shfl_xor_sync(0xffffffffu, s, 16);
+        if (idx < T.n && (!two || lane < 16)) done(R, in, s);
+    }
+}
+
+template <int FF>
+__global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
+    extern __shared__ __align__(128) unsigned char dsm[];
+    __shared__ Tables tb;
+    __shared__ __align__(8) uint64_t mbar;
+    __shared__ uint32_t tmem_base;
+    __shared__ int abort_flag, s_abort, s_chunk;
+    __shared__ double sh[NW], s_val, s_coef;
+    __shared__ float s_l[64];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned G = gridDim.x;
+    const uint32_t sm = su32(dsm), sB = sm + P.oB;
+    const int mtx = (P.px + 127) >> 7, mty = (P.py + 127) >> 7, mtz = (P.pz + 127) >> 7;
+    double *part_pq = P.part, *part_rr = P.part + G, *part_rz = P.part + 2 * G, *part_bb = P.part + 3 * G;
+    for (int i = threadIdx.x; i < 8 * ST_MAXE; i += NTH) tb.code[i] = P.code[i];
+    if (threadIdx.x < 8) tb.type[threadIdx.x] = P.types[threadIdx.x];
+    if (threadIdx.x == 0) {
+        int w = 0;
+        for (int t = 0; t < 8; ++t) { tb.wblk[t] = w; const int per = P.types[t].nent > SPLIT_ROW ? 16 : 32; w += ((int)P.types[t].n + per - 1) / per; }
+        tb.wblk[8] = w;
+        s_abort = 0;
+    }
+    load_axis<NW>(sm + P.oSt[0], P.St[0], P.px); load_axis<NW>(sm + P.oS[0], P.S[0], P.px);
+    load_axis<NW>(sm + P.oSt[1], P.St[1], P.py); load_axis<NW>(sm + P.oS[1], P.S[1], P.py);
+    load_axis<NW>(sm + P.oSt[2], P.St[2], P.pz); load_axis<NW>(sm + P.oS[2], P.S[2], P.pz);
+    Cta c;
+    cta_open(c, &mbar, &tmem_base, &abort_flag, P.tcols);
+    unsigned target = 0;
+    bool ok = true;
+
+    // r = rhs - L U, zero on the boundary, where z and p stay zero too
+    {
+        double rr = 0.0, bb = 0.0;
+        for_rows(P, tb,
+                 [&](const Row &R) {
+                     double s = 0.0;
+                     row_product(tb, R, P.val, [&](int j) { return P.V.U[j]; }, [&](double v, double x) { s = fma(v, x, s); });
+                     return s;
+                 },
+                 [&](const Row &R, bool in, double s) {
+                     if (!in) {
+                         P.V.r[R.node] = 0.0; P.p[R.node] = 0.0;
+                         if (FF) P.pf[R.node] = make_float2(0.f, 0.f);
+                         return;
+                     }
+                     const double f = P.rhs[R.node], ri = f - s;
+                     P.V.r[R.node] = ri;
+                     rr = fma(ri, ri, rr);
+                     bb = fma(f, f, bb);
+                 });
+        const double t0 = cta_sum<NW>(rr, sh);
+        __syncthreads();
+        const double t1 = cta_sum<NW>(bb, sh);
+        if (threadIdx.x == 0) { part_rr[blockIdx.x] = t0; part_bb[blockIdx.x] = t1; }
+    }
+    ok = grid_barrier(P.out, target, &s_abort);
+    const double bb = grid_total(part_bb, &s_val);
+    __syncthreads();
+    double rr = grid_total(part_rr, &s_val), rr_prev = 0.0, rz = 0.0, rate = P.rate;
+    int it = 0, it_prev = 0, status = OFKS_OK;
+
+    // the three passes; with update the CG update r -= alpha q first.  Leaves r.z's partials.
+    auto precondition = [&](bool update, double alpha) -> bool {
+        double none = 0.0, prz = 0.0;
+        bool good = true;
+        for (int a = blockIdx.x; a < P.nx && good; a += G) {
+            if (update) residual_to_data<NW, 1, 0>(P.V, a, P.ny, P.nz, P.py, P.pz, alpha, none, dsm, P.oB, P.part_p);
+            else residual_to_data<NW, 0, 0>(P.V, a, P.ny, P.nz, P.py, P.pz, alpha, none, dsm, P.oB, P.part_p);
+            good = contract(c, sm + P.oSt[2], sB, P.part_p, mtz, P.py, P.pz);
+            if (!good) break;
+            acc_to_data<NW>(c, mtz, P.py, P.pz, sB, P.part_p);
+            good = contract(c, sm + P.oSt[1], sB, P.part_p, mty, P.pz, P.py);
+            if (!good) break;
+            acc_to_global<NW>(c, mty, P.pz, P.ny, P.pz, P.T + (int64_t)a * P.ny * P.pz, P.pz);
+        }
+        if (!good && threadIdx.x == 0) { s_abort = 1; atomicExch(&P.out->abort, 1); }
+        if (!grid_barrier(P.out, target, &s_abort)) return false;
+        for (int m0 = (int)blockIdx.x * P.NT; m0 < P.ncol && good; m0 += (int)G * P.NT) {
+            mid_scales(P.lyzp, m0, P.ncol, P.NT, s_l);
+            global_to_data<NW>(P.T + m0, P.ncol, P.nx, P.ncol - m0, P.NT, P.px, sB, P.part_m);
+            good = contract(c, sm + P.oSt[0], sB, P.part_m, mtx, P.NT, P.px);
+            if (!good) break;
+            mid_scale<NW>(c, mtx, P.NT, P.nx, P.px, P.lx, s_l, dsm, P.oB, P.part_m);
+            good = contract(c, sm + P.oS[0], sB, P.part_m, mtx, P.NT, P.px);
+            if (!good) break;
+            acc_to_global<NW>(c, mtx, P.NT, P.nx, P.ncol - m0, P.T + m0, P.ncol);
+        }
+        if (!good && threadIdx.x == 0) { s_abort = 1; atomicExch(&P.out->abort, 1); }
+        if (!grid_barrier(P.out, target, &s_abort)) return false;
+        for (int a = blockIdx.x; a < P.nx && good; a += G) {
+            global_to_data<NW>(P.T + (int64_t)a * P.ny * P.pz, P.pz, P.ny, P.pz, P.pz, P.py, sB, P.part_p);
+            good = contract(c, sm + P.oS[1], sB, P.part_p, mty, P.pz, P.py);
+            if (!good) break;
+            acc_to_data<NW>(c, mty, P.pz, P.py, sB, P.part_p);
+            good = contract(c, sm + P.oS[2], sB, P.part_p, mtz, P.py, P.pz);
+            if (!good) break;
+            acc_to_z<NW, 1>(c, mtz, P.V, a, P.ny, P.nz, P.py, P.zf, nullptr, nullptr, prz);
+        }
+        const double t = cta_sum<NW>(prz, sh);
+        if (threadIdx.x == 0) part_rz[blockIdx.x] = t;
+        if (!good && threadIdx.x == 0) { s_abort = 1; atomicExch(&P.out->abort, 1); }
+        return grid_barrier(P.out, target, &s_abort);
+    };
+    // U += alpha p, p = z + beta p and r.r on the interior (warps over the rows along c), spread over
+    // the whole grid: the passes over planes run on as many CTAs as there are planes, and every
+    // float64 operation of a warp takes 16 cycles
+    auto direction = [&](double alpha, double beta) {
+        double prr = 0.0;
+        for (int row = warp * G + blockIdx.x; row < P.nx * P.ny; row += NW * G) {
+            const int a = row / P.ny, b = row - a * P.ny;
+            const int o = ((a + 1) * P.V.Ly + (b + 1)) * P.V.Lz + 1;
+            for (int cc = lane; cc < P.nz; cc += 32) {
+                const double pv = P.p[o + cc], zv = f2d_bits(P.zf[o + cc]), rv = P.V.r[o + cc];
+                if (alpha != 0.0) P.V.U[o + cc] = fma(alpha, pv, P.V.U[o + cc]);
+                const double v = beta != 0.0 ? fma(beta, pv, zv) : zv;
+                P.p[o + cc] = v;
+                if (FF) P.pf[o + cc] = ff_split(v);
+                prr = fma(rv, rv, prr);
+            }
+        }
+        prr = cta_sum<NW>(prr, sh);
+        if (threadIdx.x == 0) part_rr[blockIdx.x] = prr;
+    };
+
+    while (ok) {
+        // the residual test, and the iterations to the next one: the count that the last observed
+        // factor of the squared residual predicts to the target, 1 to 8 (4 before any is known)
+        if (!isfinite(rr)) { status = OFKS_ENONFINITE; break; }
+        if (rr <= P.tol2 * bb || bb == 0.0) {
+            if (it > it_prev && rr_prev > 0.0 && rr > 0.0 && rr < rr_prev) rate = pow(rr / rr_prev, 1.0 / (it - it_prev));
+            break;
+        }
+        if (it >= P.max_iter) { status = OFKS_ETIMEOUT; break; }
+        if (threadIdx.x == 0) {
+            double f = rate;
+            if (it > 0 && rr_prev > 0.0 && rr < rr_prev) f = pow(rr / rr_prev, 1.0 / (it - it_prev));
+            int chunk = 4;
+            if (f > 0.0 && f < 1.0) {
+                const double need = log(P.tol2 * bb / rr) / log(f);
+                chunk = (int)fmin(8.0, fmax(1.0, ceil(need)));
+            } else {
+                f = rate;
+            }
+            s_chunk = chunk;
+            s_coef = f;
+        }
+        __syncthreads();
+        const int chunk = s_chunk;
+        rate = s_coef;
+        rr_prev = rr;
+        it_prev = it;
+        if (it == 0) {                            // z = A_sep^-1 r, p = z
+            ok = precondition(false, 0.0);
+            if (!ok) break;
+            rz = grid_total(part_rz, &s_val);
+            direction(0.0, 0.0);
+            ok = grid_barrier(P.out, target, &s_abort);
+        }
+        for (int j = 0; j < chunk && ok; ++j) {
+            double pq = 0.0;
+            for_rows(P, tb,
+                     [&](const Row &R) {
+                         if constexpr (FF) {
+                             float s_hi = 0.f, s_lo = 0.f;
+                             row_product(tb, R, P.valff, [&](int i) { return P.pf[i]; },
+                                         [&](float2 v, float2 x) { ff_madd(s_hi, s_lo, v, x); });
+                             return (double)s_hi + (double)s_lo;
+                         } else {
+                             double s = 0.0;
+                             row_product(tb, R, P.val, [&](int i) { return P.p[i]; },
+                                         [&](double v, double x) { s = fma(v, x, s); });
+                             return s;
+                         }
+                     },
+                     [&](const Row &R, bool in, double s) {
+                         if (!in) return;
+                         P.q[R.node] = s;
+                         pq = fma(P.p[R.node], s, pq);
+                     });
+            const double tpq = cta_sum<NW>(pq, sh);
+            if (threadIdx.x == 0) part_pq[blockIdx.x] = tpq;
+            if (!(ok = grid_barrier(P.out, target, &s_abort))) break;
+            const double den = grid_total(part_pq, &s_val);
+            if (threadIdx.x == 0) s_coef = den > 0.0 ? rz / den : 0.0;
+            __syncthreads();
+            const double alpha = s_coef;
+            if (!(ok = precondition(true, alpha))) break;
+            const double rz2 = grid_total(part_rz, &s_val);
+            if (threadIdx.x == 0) s_coef = rz > 0.0 ? rz2 / rz : 0.0;
+            __syncthreads();
+            const double beta = s_coef;
+            rz = rz2;
+            direction(alpha, beta);
+            ok = grid_barrier(P.out, target, &s_abort);
+            ++it;
+        }
+        if (ok) rr = grid_total(part_rr, &s_val);
+        __syncthreads();
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        P.out->rr = rr; P.out->bb = bb; P.out->rate = rate; P.out->it = it; P.out->status = status;
+    }
+    cta_close(c, P.tcols, &P.out->abort);
+}
+
+// shared memory of the loop kernel; 0 when the operands do not fit
+int place_loop(const SepState &S, Loop &P) {
+    P.nx = S.n[0]; P.ny = S.n[1]; P.nz = S.n[2];
+    P.px = pad16(P.nx); P.py = pad16(P.ny); P.pz = pad16(P.nz);
+    P.ncol = P.ny * P.pz;
+    P.NT = (P.ncol + 31) / 32 >= 100 ? ((P.ncol + 63) / 64 >= 120 ? 64 : 32) : 16;
+    const int pad[3] = {P.px, P.py, P.pz};
+    uint32_t o = 0;
+    for (int d = 0; d < 3; ++d) {
+        P.S[d] = S.hS[d]; P.St[d] = S.hSt[d];
+        P.oSt[d] = o; o += axis_bytes(pad[d]);
+        P.oS[d] = o; o += axis_bytes(pad[d]);
+    }
+    P.oB = o;
+    P.part_p = data_bytes(P.py, P.pz);
+    P.part_m = data_bytes(P.NT, P.px);
+    P.lx = S.lx; P.lyzp = S.lyzp; P.T = S.t0;
+    P.tcols = cols_of(std::max({tiles128(P.px) * P.NT, tiles128(P.pz) * P.py, tiles128(P.py) * P.pz}));
+    const uint32_t need = o + 2 * std::max(P.part_p, P.part_m);
+    return need <= (uint32_t)(SMEM_MAX - 20 * 1024) && P.tcols <= 512 ? (int)need : 0;
+}
+
+}  // namespace
+
+// room for the result record and the partials
+int64_t cg_loop_doubles(int sms) { return 8 + 4 * (int64_t)sms; }
+
+// the persistent form applies: its operands fit in an SM's shared memory (axes of about 100
+// interior points) and the mesh is small enough for launches to matter
+bool cg_loop_fits(const SepState &S) {
+    Loop P{};
+    return S.plane && (int64_t)S.n[0] * S.n[1] * S.n[2] <= CG_LOOP_MAX_N && place_loop(S, P) > 0;
+}
+
+// Solves L U = rhs on the interior from U's current values and boundary data to
+// |r|^2 <= tol2 |rhs|^2; iterations and status (OFKS_OK, OFKS_ETIMEOUT at max_iter,
+// OFKS_ENONFINITE, or an error) on return.  One launch, one synchronization.
+int cg_loop_run(ofks_ctx *c, double tol2, int *iters, int *status, double *rel2) {
+    SepState &S = c->sep;
+    Loop P{};
+    const int smem = place_loop(S, P);
+    P.V = {c->st.Ly, c->st.Lz, c->d_cp, c->d_cq, c->d_U, c->d_cr, c->d_cz};
+    P.p = c->d_cp; P.zf = reinterpret_cast<float *>(c->d_cz); P.q = c->d_cq; P.pf = c->hartree_ff ? c->d_cpff : nullptr; P.rhs = c->d_rhs;
+    P.Lx = c->st.Lx;
+    P.types = c->st.d_type; P.code = c->st.d_code; P.val = c->st.val; P.valff = c->st.valff;
+    P.tol2 = tol2; P.rate = c->cg_rate; P.max_iter = c->prm.poisson_max_iter;
+    P.out = reinterpret_cast<CgOut *>(S.loop_buf);
+    P.part = S.loop_buf + 8;
+    // CTAs: one per SM, fewer where the mesh has too few planes, tiles and rows to feed them
+    const int64_t rows = c->n_nodes;
+    const int want = std::max({P.nx, (P.ncol + P.NT - 1) / P.NT, (int)std::min<int64_t>(1 << 20, (rows + NTH - 1) / NTH)});
+    const int grid = std::min(S.sms, want);
+    auto kern = c->hartree_ff ? k_cg_loop<1> : k_cg_loop<0>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaMemsetAsync(S.loop_buf, 0, sizeof(double) * 8, c->stream);
+    void *args[] = {&P};
+    if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)grid), dim3(NTH), args, smem, c->stream);
+    c->kernels += 1;
+    CgOut h;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, P.out, sizeof(h), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return ofks_cuda_check(c, e, "Hartree CG");
+    if (h.abort) return ofks_fail(c, OFKS_ETIMEOUT, "Hartree CG: a bounded device wait timed out");
+    c->cg_rate = h.rate;
+    *iters = h.it;
+    *status = h.status;
+    *rel2 = h.bb > 0.0 ? h.rr / h.bb : 0.0;
+    return OFKS_OK;
+}

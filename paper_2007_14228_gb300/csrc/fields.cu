@@ -565,6 +565,29 @@ int run_hartree(ofks_ctx *c) {
     k_boundary<<<(c->n_bnd + 255) / 256, 256, 0, c->stream>>>(c->n_bnd, c->d_bnd, c->d_bxyz,
                                                                c->d_sc + SC_MOM, c->prm.multipole_lmax,
                                                                c->d_U);
+    double ptol = c->phase == 32 ? std::max(c->prm.poisson_tol, c->prm.poisson_tol_mixed) : c->prm.poisson_tol;
+    if (c->hartree_tol > 0.0) ptol = std::max(ptol, c->hartree_tol);
+    const double tol2 = ptol * ptol;
+    const int pc = hartree_pc(c);
+    const bool amg = pc != OFKS_HPC_JACOBI;             // a preconditioner other than the diagonal
+    const bool sep = pc == OFKS_HPC_SEPARABLE;
+    const bool lat = c->st.on && !c->prm.poisson_csr;
+    // during the float32 iterations the lattice SpMV of the separable CG runs in float-float
+    // arithmetic (~48 bits, its tolerance is at least poisson_tol_mixed); float64 otherwise
+    c->hartree_ff = sep && lat && c->phase == 32 && c->st.valff != nullptr;
+    if (sep && lat && c->sep.loop && c->prm.poisson_sep_tc) {
+        int iters = 0, status = OFKS_OK;
+        double rel2 = 0.0;
+        c->kernels += 1;
+        const int rc = cg_loop_run(c, tol2, &iters, &status, &rel2);
+        if (rc) return rc;
+        if (status == OFKS_ENONFINITE) return ofks_fail(c, status, "Hartree CG residual is not finite");
+        if (status == OFKS_ETIMEOUT)
+            return ofks_fail(c, status, "Hartree CG: %d iterations, relative residual %.3e", iters, std::sqrt(rel2));
+        c->cg_last = iters;
+        c->cg_total += iters;
+        return OFKS_OK;
+    }
     cudaMemsetAsync(sc, 0, sizeof(double) * 8, c->stream);
     if (c->st.on && !c->prm.poisson_csr) {   // the lattice-stencil residual, then the CG start
         launch_stencil_residual(c, c->d_U, c->d_rhs, c->d_cr);
@@ -575,17 +598,10 @@ int run_hartree(ofks_ctx *c) {
                                              c->d_cr, c->d_cz, c->d_cp, sc, c->d_gpart, c->d_gcount);
     }
     c->kernels += 2;
-    const int pc = hartree_pc(c);
-    const bool amg = pc != OFKS_HPC_JACOBI;             // a preconditioner other than the diagonal
     auto precond = [&]() {
         ProfScope pp(c, PF_POISSON_PC);
         amg_apply(c, c->d_cr, c->d_cz);
     };
-    const bool sep = pc == OFKS_HPC_SEPARABLE;
-    const bool lat = c->st.on && !c->prm.poisson_csr;
-    // during the float32 iterations the lattice SpMV of the separable CG runs in float-float
-    // arithmetic (~48 bits, its tolerance is at least poisson_tol_mixed); float64 otherwise
-    c->hartree_ff = sep && lat && c->phase == 32 && c->st.valff != nullptr;
     auto spmv = [&](int it) {
         ProfScope pv(c, PF_POISSON_SPMV);
         if (lat) { launch_stencil_spmv(c, c->d_cp, c->d_cq, sc, it); return; }
@@ -603,9 +619,6 @@ int run_hartree(ofks_ctx *c) {
         k_cg_rz<<<gU, 256, 0, c->stream>>>(N, c->d_cr, c->d_cz, c->d_cp, sc, 0, 1, c->d_gpart, c->d_gcount);
         c->kernels += 1;
     }
-    double ptol = c->phase == 32 ? std::max(c->prm.poisson_tol, c->prm.poisson_tol_mixed) : c->prm.poisson_tol;
-    if (c->hartree_tol > 0.0) ptol = std::max(ptol, c->hartree_tol);
-    const double tol2 = ptol * ptol;
     int chunk = amg ? 4 : 32;
     int it = 0, it_prev = 0;
     double h[8], rr_prev = 0.0;

@@ -94,6 +94,15 @@ struct StencilEntry {
     int8_t oa, ob, oc, tp;                       // lattice offset; source type (-1: own slot)
     int slot;                                    // slot in the source type
 };
+// Compact form of an entry: value index off + (index of (ia, ib, ic) in a sub-lattice whose extents
+// have the parities `cls`), neighbour id row + lin.  For a row with sub-lattice coordinates
+// (ia, ib, ic) that index is (ia ny + ib) nz + ic, where ny and nz are those of the parity class
+// (cls bit 1: odd along the second axis, bit 0: odd along the third), so a row computes four
+// indices once and an entry costs one shared load, a selection and two additions.
+struct StencilCode {
+    int64_t off;
+    int lin4, pad;                               // lin 4 + cls
+};
 struct Stencil {
     bool on = false;
     int Lx = 0, Ly = 0, Lz = 0, blocks = 0;
@@ -101,7 +110,7 @@ struct Stencil {
     double *val = nullptr;
     float2 *valff = nullptr;                     // val as float32 pairs (float-float SpMV)
     StencilType *d_type = nullptr;
-    StencilEntry *d_ent = nullptr;               // 8 x ST_MAXE
+    StencilCode *d_code = nullptr;               // 8 x ST_MAXE
     int *d_slot = nullptr;                       // 8 x 125 offset code -> own slot or -1
 };
 
@@ -112,7 +121,12 @@ struct SepState {
     float *S[3] = {nullptr, nullptr, nullptr};   // per-axis modes S[a][i] (n x n)
     float *St[3] = {nullptr, nullptr, nullptr};  // their transposes
     float *lx = nullptr, *lyz = nullptr;         // lam_x (nx), lam_y + lam_z (ny x nz)
-    float *t0 = nullptr, *t1 = nullptr;          // interior tensors
+    float *lyzp = nullptr;                       // lyz with rows of nz rounded up to 16 (padding 1e30)
+    float *t0 = nullptr, *t1 = nullptr;          // interior tensors (t0 also with padded rows)
+    bool plane = false;                          // the three-pass form applies (sep_plane.cu)
+    bool loop = false;                           // the persistent form of the CG applies (cg_loop.cu)
+    int sms = 0;                                 // SMs of the device
+    double *loop_buf = nullptr;                  // its result record and reduction partials
     bool tc = false;                             // tensor-core form available (every axis <= 256)
     __nv_bfloat16 *hS[3] = {nullptr, nullptr, nullptr}, *hSt[3] = {nullptr, nullptr, nullptr};  // bf16, padded
     __nv_bfloat16 *hbuf = nullptr;               // six padded bf16 tensors (input, intermediates)
@@ -310,6 +324,16 @@ void sep_cg_step(ofks_ctx *c, int it, int slot, int first);    // fused CG updat
 void sep_free(ofks_ctx *c);
 bool sep_pcg_ready(ofks_ctx *c, int w);                        // separable PCG buffers for width w
 void sep_pcg_passes(ofks_ctx *c, int w, const double *shift);  // z = T_sep^-1 r on the PCG tensor
+// the Hartree step in three passes (sep_plane.cu)
+bool sep_plane_fits(const SepState &S);
+// The whole Hartree CG as one persistent kernel (cg_loop.cu), up to CG_LOOP_MAX_N interior nodes: on
+// the largest meshes that its shared memory admits beyond that, the SpMV at one CTA per SM loses
+// against its own kernel at full occupancy what the launches cost.
+constexpr int64_t CG_LOOP_MAX_N = 600000;
+bool cg_loop_fits(const SepState &S);
+int64_t cg_loop_doubles(int sms);
+int cg_loop_run(ofks_ctx *c, double tol2, int *iters, int *status, double *rel2);
+void sep_plane_hartree(ofks_ctx *c, int it, int slot, int first);
 
 // ---- fields.cu (density, potentials, Hamiltonian refresh, Poisson)
 int hartree_pc(ofks_ctx *c);                    // OFKS_HPC_* the next Hartree solve uses (builds the

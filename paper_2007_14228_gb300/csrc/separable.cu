@@ -486,8 +486,9 @@ inline int pad16(int x) { return (x + 15) / 16 * 16; }
 
 void sep_free(ofks_ctx *c) {
     SepState &S = c->sep;
-    for (float *p : {S.S[0], S.S[1], S.S[2], S.St[0], S.St[1], S.St[2], S.lx, S.lyz, S.t0, S.t1})
+    for (float *p : {S.S[0], S.S[1], S.S[2], S.St[0], S.St[1], S.St[2], S.lx, S.lyz, S.lyzp, S.t0, S.t1})
         if (p) cudaFree(p);
+    if (S.loop_buf) cudaFree(S.loop_buf);
     for (void *p : {(void *)S.hS[0], (void *)S.hS[1], (void *)S.hS[2], (void *)S.hSt[0], (void *)S.hSt[1],
                     (void *)S.hSt[2], (void *)S.hbuf, (void *)S.hlo, (void *)S.pbuf})
         if (p) cudaFree(p);
@@ -539,8 +540,13 @@ int sep_setup(ofks_ctx *c, const double *xyz, const uint8_t *dirichlet) {
     }
     upf(&S.lx, lx);
     upf(&S.lyz, lyz);
-    // tensor-core operands: bf16 axis matrices padded to multiples of 16, and five zeroed
-    // intermediate tensors whose innermost axis is padded the same way
+    std::vector<float> lyzp((size_t)n[1] * pad16(n[2]), 1e30f);
+    for (int j = 0; j < n[1]; ++j)
+        for (int k = 0; k < n[2]; ++k) lyzp[(size_t)j * pad16(n[2]) + k] = lyz[(size_t)j * n[2] + k];
+    upf(&S.lyzp, lyzp);
+    S.n[0] = n[0]; S.n[1] = n[1]; S.n[2] = n[2];
+    // tensor-core operands: bf16 axis matrices padded to multiples of 16, and for the six-pass form
+    // six zeroed tensors whose innermost axis is padded the same way
     S.tc = n[0] <= 256 && n[1] <= 256 && n[2] <= 256;
     if (S.tc && e == cudaSuccess) {
         for (int d = 0; d < 3; ++d) {
@@ -558,24 +564,28 @@ int sep_setup(ofks_ctx *c, const double *xyz, const uint8_t *dirichlet) {
                 if (e == cudaSuccess) e = cudaMemcpy(*dst, h.data(), sizeof(__nv_bfloat16) * h.size(), cudaMemcpyHostToDevice);
             }
         }
+        S.plane = sep_plane_fits(S);
         // [a][b][c~], [k][a][b~], [j][k][a~], [i][j][k~], [c][i][j~], [b][c][i~]  (~ = padded to 16)
         const int64_t len[6] = {(int64_t)n[0] * n[1] * pad16(n[2]), (int64_t)n[2] * n[0] * pad16(n[1]),
                                 (int64_t)n[1] * n[2] * pad16(n[0]), (int64_t)n[0] * n[1] * pad16(n[2]),
                                 (int64_t)n[2] * n[0] * pad16(n[1]), (int64_t)n[1] * n[2] * pad16(n[0])};
         int64_t tot = 0;
         for (int q = 0; q < 6; ++q) { S.hoff[q] = tot; tot += (len[q] + 63) / 64 * 64; }
-        if (e == cudaSuccess) e = cudaMalloc((void **)&S.hbuf, sizeof(__nv_bfloat16) * tot);
-        if (e == cudaSuccess) e = cudaMemset(S.hbuf, 0, sizeof(__nv_bfloat16) * tot);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&S.hlo, sizeof(__nv_bfloat16) * tot);
-        if (e == cudaSuccess) e = cudaMemset(S.hlo, 0, sizeof(__nv_bfloat16) * tot);
+        for (__nv_bfloat16 **q : {&S.hbuf, &S.hlo}) {
+            if (S.plane) break;
+            if (e == cudaSuccess) e = cudaMalloc((void **)q, sizeof(__nv_bfloat16) * tot);
+            if (e == cudaSuccess) e = cudaMemset(*q, 0, sizeof(__nv_bfloat16) * tot);
+        }
     }
-    if (e == cudaSuccess) e = cudaMalloc((void **)&S.t0, sizeof(float) * nt);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&S.t0, sizeof(float) * ((size_t)n[0] * n[1] * pad16(n[2])));
     if (e == cudaSuccess) e = cudaMalloc((void **)&S.t1, sizeof(float) * nt);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&S.sms, cudaDevAttrMultiProcessorCount, c->device);
+    S.loop = e == cudaSuccess && cg_loop_fits(S);
+    if (S.loop) e = cudaMalloc((void **)&S.loop_buf, sizeof(double) * cg_loop_doubles(S.sms));
     if (e != cudaSuccess) {
         sep_free(c);
         return ofks_fail(c, OFKS_ENOMEM, "set_mesh: separable preconditioner: %s", cudaGetErrorString(e));
     }
-    S.n[0] = n[0]; S.n[1] = n[1]; S.n[2] = n[2];
     S.on = true;
     if (std::getenv("OFKS_VERBOSE"))
         std::fprintf(stderr, "[ofks sep] interior %d x %d x %d, lam_x in [%.3e, %.3e]\n", n[0], n[1], n[2],
@@ -592,6 +602,10 @@ void sep_cg_step(ofks_ctx *c, int it, int slot, int first) {
     const int64_t nt = (int64_t)nx * ny * nz;
     const unsigned g = (unsigned)std::min<int64_t>((nt + 255) / 256, 152 * 8);
     double *sc = c->d_sc + SC_CG;
+    if (S.plane && c->prm.poisson_sep_tc) {
+        sep_plane_hartree(c, it, slot, first);
+        return;
+    }
     if (S.tc && c->prm.poisson_sep_tc) {
         // every tensor as a high and a low bf16 part: the rounding of the intermediates to 8 bits
         // made the preconditioner visibly nonlinear and cost the CG about a quarter more iterations

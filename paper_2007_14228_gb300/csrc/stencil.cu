@@ -47,6 +47,21 @@ __global__ void k_st_fill(int64_t N, int Ly, int Lz, const int *__restrict__ fpt
     }
 }
 
+// index of (ia, ib, ic) in the sub-lattices of the four parity classes, and the one an entry asks for
+// (StencilCode): the addressing of an entry was ~30 instructions with the type tables, more than its
+// arithmetic in the float-float form
+__device__ __forceinline__ int4 class_index(int Ly, int Lz, int ia, int ib, int ic) {
+    const int y0 = (Ly + 1) >> 1, y1 = Ly >> 1, z0 = (Lz + 1) >> 1, z1 = Lz >> 1;
+    const int r0 = ia * y0 + ib, r1 = ia * y1 + ib;
+    return make_int4(r0 * z0 + ic, r0 * z1 + ic, r1 * z0 + ic, r1 * z1 + ic);
+}
+__device__ __forceinline__ int of_class(const int4 cl, int lin4) {
+    const int lo = lin4 & 1 ? cl.y : cl.x, hi = lin4 & 1 ? cl.w : cl.z;
+    return lin4 & 2 ? hi : lo;
+}
+
+constexpr int ST_B = 4;                           // entries whose loads are issued together (float64)
+
 // Row sums s_i = (L x)_i over the non-Dirichlet rows, then by MODE
 //   0: y = s and pq += x.s (slot it&1), zeroing the retired rz / rr slots (the CG protocol of
 //      the CSR kernel)
@@ -56,20 +71,20 @@ __global__ void k_st_fill(int64_t N, int Ly, int Lz, const int *__restrict__ fpt
 // row, and every lane of a warp runs the same stencil.  Dirichlet rows are not written.
 template <int MODE>
 __global__ void __launch_bounds__(256) k_st_apply(int Ly, int Lz, const StencilType *__restrict__ types,
-                                                  const StencilEntry *__restrict__ ents,
+                                                  const StencilCode *__restrict__ code,
                                                   const double *__restrict__ val, const double *__restrict__ minv,
                                                   const double *__restrict__ xv, const double *__restrict__ bv,
                                                   double w, double *yv, double *sc, int it, double *gpart,
                                                   unsigned *gcount) {
     __shared__ StencilType st[8];
-    __shared__ StencilEntry se[ST_MAXE];
+    __shared__ StencilCode se[ST_MAXE];
     __shared__ double sh[8];
     if (threadIdx.x < 8) st[threadIdx.x] = types[threadIdx.x];
     __syncthreads();
     int t = 0;
     while (t < 7 && (int)blockIdx.x >= st[t + 1].blk0) ++t;
     const StencilType T = st[t];
-    for (int e = threadIdx.x; e < T.nent; e += blockDim.x) se[e] = ents[t * ST_MAXE + e];
+    for (int e = threadIdx.x; e < T.nent; e += blockDim.x) se[e] = code[t * ST_MAXE + e];
     __syncthreads();
     const int64_t idx = (int64_t)((int)blockIdx.x - T.blk0) * blockDim.x + threadIdx.x;
     double pq = 0.0;
@@ -82,19 +97,23 @@ __global__ void __launch_bounds__(256) k_st_apply(int Ly, int Lz, const StencilT
         const int64_t row = ((int64_t)a * Ly + b) * Lz + c;
         const double mi = minv[row];
         if (mi != 0.0) {
+            const int4 cl = class_index(Ly, Lz, ia, ib, ic);
             double s = 0.0;
             int e = 0;
-#pragma unroll 4
-            for (; e < T.nown; ++e) {   // stored with this row
-                const StencilEntry E = se[e];
-                s = fma(val[T.base + (int64_t)E.slot * T.n + idx], xv[row + E.lin], s);
+            for (; e + ST_B <= T.nent; e += ST_B) {
+                double v[ST_B], x[ST_B];
+#pragma unroll
+                for (int u = 0; u < ST_B; ++u) {
+                    const StencilCode E = se[e + u];
+                    v[u] = val[E.off + of_class(cl, E.lin4)];
+                    x[u] = xv[row + (E.lin4 >> 2)];
+                }
+#pragma unroll
+                for (int u = 0; u < ST_B; ++u) s = fma(v[u], x[u], s);
             }
-#pragma unroll 4
-            for (; e < T.nent; ++e) {   // stored with the neighbour (symmetric half)
-                const StencilEntry E = se[e];
-                const StencilType &S = st[E.tp];
-                const int64_t j = ((int64_t)((a + E.oa) >> 1) * S.ny + ((b + E.ob) >> 1)) * S.nz + ((c + E.oc) >> 1);
-                s = fma(val[S.base + (int64_t)E.slot * S.n + j], xv[row + E.lin], s);
+            for (; e < T.nent; ++e) {
+                const StencilCode E = se[e];
+                s = fma(val[E.off + of_class(cl, E.lin4)], xv[row + (E.lin4 >> 2)], s);
             }
             if (MODE == 0) { yv[row] = s; pq = xv[row] * s; }
             else if (MODE == 1) yv[row] = bv[row] - s;
@@ -134,20 +153,20 @@ __device__ __forceinline__ void ff_madd(float &sh, float &sl, const float2 a, co
 constexpr int FF_B = 8;                           // entries whose loads are issued together
 
 __global__ void __launch_bounds__(256) k_st_apply_ff(int Ly, int Lz, const StencilType *__restrict__ types,
-                                                     const StencilEntry *__restrict__ ents,
+                                                     const StencilCode *__restrict__ code,
                                                      const float2 *__restrict__ val, const double *__restrict__ minv,
                                                      const float2 *__restrict__ xf, const double *__restrict__ xv,
                                                      double *yv, double *sc, int it, double *gpart,
                                                      unsigned *gcount) {
     __shared__ StencilType st[8];
-    __shared__ StencilEntry se[ST_MAXE];
+    __shared__ StencilCode se[ST_MAXE];
     __shared__ double sh[8];
     if (threadIdx.x < 8) st[threadIdx.x] = types[threadIdx.x];
     __syncthreads();
     int t = 0;
     while (t < 7 && (int)blockIdx.x >= st[t + 1].blk0) ++t;
     const StencilType T = st[t];
-    for (int e = threadIdx.x; e < T.nent; e += blockDim.x) se[e] = ents[t * ST_MAXE + e];
+    for (int e = threadIdx.x; e < T.nent; e += blockDim.x) se[e] = code[t * ST_MAXE + e];
     __syncthreads();
     const int64_t idx = (int64_t)((int)blockIdx.x - T.blk0) * blockDim.x + threadIdx.x;
     double pq = 0.0;
@@ -160,27 +179,23 @@ __global__ void __launch_bounds__(256) k_st_apply_ff(int Ly, int Lz, const Stenc
         const int64_t row = ((int64_t)a * Ly + b) * Lz + c;
         if (minv[row] != 0.0) {
             float s_hi = 0.f, s_lo = 0.f;
-            // entry e's value: own slots (e < nown) at this row's index, mirrored ones at the
-            // neighbour's index in its type's arrays
-            auto vaddr = [&](int e) -> const float2 * {
-                const StencilEntry E = se[e];
-                if (e < T.nown) return val + T.base + (int64_t)E.slot * T.n + idx;
-                const StencilType &S = st[E.tp];
-                const int64_t j = ((int64_t)((a + E.oa) >> 1) * S.ny + ((b + E.ob) >> 1)) * S.nz + ((c + E.oc) >> 1);
-                return val + S.base + (int64_t)E.slot * S.n + j;
-            };
+            const int4 cl = class_index(Ly, Lz, ia, ib, ic);
             int e = 0;
             for (; e + FF_B <= T.nent; e += FF_B) {
                 float2 v[FF_B], x[FF_B];
 #pragma unroll
                 for (int u = 0; u < FF_B; ++u) {
-                    v[u] = __ldg(vaddr(e + u));
-                    x[u] = __ldg(xf + row + se[e + u].lin);
+                    const StencilCode E = se[e + u];
+                    v[u] = __ldg(val + E.off + of_class(cl, E.lin4));
+                    x[u] = __ldg(xf + row + (E.lin4 >> 2));
                 }
 #pragma unroll
                 for (int u = 0; u < FF_B; ++u) ff_madd(s_hi, s_lo, v[u], x[u]);
             }
-            for (; e < T.nent; ++e) ff_madd(s_hi, s_lo, __ldg(vaddr(e)), __ldg(xf + row + se[e].lin));
+            for (; e < T.nent; ++e) {
+                const StencilCode E = se[e];
+                ff_madd(s_hi, s_lo, __ldg(val + E.off + of_class(cl, E.lin4)), __ldg(xf + row + (E.lin4 >> 2)));
+            }
             const double s = (double)s_hi + (double)s_lo;
             yv[row] = s;
             pq = xv[row] * s;
@@ -202,7 +217,8 @@ __global__ void k_st_split(int64_t len, const double *__restrict__ v, float2 *vf
 }  // namespace
 
 void stencil_free(ofks_ctx *c) {
-    cudaFree(c->st.val); cudaFree(c->st.valff); cudaFree(c->st.d_type); cudaFree(c->st.d_ent); cudaFree(c->st.d_slot);
+    cudaFree(c->st.val); cudaFree(c->st.valff); cudaFree(c->st.d_type); cudaFree(c->st.d_slot);
+    cudaFree(c->st.d_code);
     c->st = Stencil{};
 }
 
@@ -331,16 +347,29 @@ int stencil_setup(ofks_ctx *c, int64_t N, const double *xyz, const int64_t *fptr
     for (unsigned w = 0; w < nt; ++w)
         if (out[w]) return OFKS_OK;
 
+    // compact entries: the value index of row (ia, ib, ic) is base + slot n + the index of
+    // (ia, ib, ic) shifted by the neighbour's sub-lattice offset, with the neighbour type's extents
+    std::vector<StencilCode> code(8 * ST_MAXE, StencilCode{0, 0, 0});
+    for (int t = 0; t < 8; ++t)
+        for (int e = 0; e < types[t].nent; ++e) {
+            const StencilEntry &E = ents[t * ST_MAXE + e];
+            const StencilType &T = types[t], &S = types[E.tp < 0 ? t : E.tp];
+            int64_t sh = 0;
+            if (E.tp >= 0)                        // floor halves: C++ shifts of negative values are arithmetic
+                sh = ((int64_t)((T.px + E.oa) >> 1) * S.ny + ((T.py + E.ob) >> 1)) * S.nz + ((T.pz + E.oc) >> 1);
+            code[t * ST_MAXE + e] = {S.base + (int64_t)E.slot * S.n + sh, E.lin * 4 + (S.py << 1 | S.pz), 0};
+        }
+
     Stencil &S = c->st;
     cudaError_t e = cudaMalloc(&S.val, sizeof(double) * std::max<int64_t>(len, 1));
     if (e == cudaSuccess) e = cudaMalloc(&S.valff, sizeof(float2) * std::max<int64_t>(len, 1));
     if (e == cudaSuccess) e = cudaMalloc(&S.d_type, sizeof(types));
-    if (e == cudaSuccess) e = cudaMalloc(&S.d_ent, sizeof(StencilEntry) * ents.size());
     if (e == cudaSuccess) e = cudaMalloc(&S.d_slot, sizeof(int) * slot.size());
+    if (e == cudaSuccess) e = cudaMalloc(&S.d_code, sizeof(StencilCode) * code.size());
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(S.d_code, code.data(), sizeof(StencilCode) * code.size(), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(S.val, 0, sizeof(double) * std::max<int64_t>(len, 1), c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(S.d_type, types, sizeof(types), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(S.d_ent, ents.data(), sizeof(StencilEntry) * ents.size(), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(S.d_slot, slot.data(), sizeof(int) * slot.size(), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -371,28 +400,28 @@ void stencil_fill(ofks_ctx *c) {
 }
 
 void launch_stencil_spmv(ofks_ctx *c, const double *p, double *q, double *sc, int it) {
-    k_st_apply<0><<<(unsigned)c->st.blocks, 256, 0, c->stream>>>(c->st.Ly, c->st.Lz, c->st.d_type, c->st.d_ent,
+    k_st_apply<0><<<(unsigned)c->st.blocks, 256, 0, c->stream>>>(c->st.Ly, c->st.Lz, c->st.d_type, c->st.d_code,
                                                                 c->st.val, c->d_minv, p, nullptr, 0.0, q, sc, it,
                                                                 c->d_gpart, c->d_gcount);
     c->kernels += 1;
 }
 
 void launch_stencil_spmv_ff(ofks_ctx *c, const float2 *pf, const double *p, double *q, double *sc, int it) {
-    k_st_apply_ff<<<(unsigned)c->st.blocks, 256, 0, c->stream>>>(c->st.Ly, c->st.Lz, c->st.d_type, c->st.d_ent,
+    k_st_apply_ff<<<(unsigned)c->st.blocks, 256, 0, c->stream>>>(c->st.Ly, c->st.Lz, c->st.d_type, c->st.d_code,
                                                                 c->st.valff, c->d_minv, pf, p, q, sc, it, c->d_gpart,
                                                                 c->d_gcount);
     c->kernels += 1;
 }
 
 void launch_stencil_residual(ofks_ctx *c, const double *x, const double *b, double *r) {
-    k_st_apply<1><<<(unsigned)c->st.blocks, 256, 0, c->stream>>>(c->st.Ly, c->st.Lz, c->st.d_type, c->st.d_ent,
+    k_st_apply<1><<<(unsigned)c->st.blocks, 256, 0, c->stream>>>(c->st.Ly, c->st.Lz, c->st.d_type, c->st.d_code,
                                                                 c->st.val, c->d_minv, x, b, 0.0, r, nullptr, 0,
                                                                 nullptr, nullptr);
     c->kernels += 1;
 }
 
 void launch_stencil_jacobi(ofks_ctx *c, const double *x, const double *b, double w, double *y) {
-    k_st_apply<2><<<(unsigned)c->st.blocks, 256, 0, c->stream>>>(c->st.Ly, c->st.Lz, c->st.d_type, c->st.d_ent,
+    k_st_apply<2><<<(unsigned)c->st.blocks, 256, 0, c->stream>>>(c->st.Ly, c->st.Lz, c->st.d_type, c->st.d_code,
                                                                 c->st.val, c->d_minv, x, b, w, y, nullptr, 0,
                                                                 nullptr, nullptr);
     c->kernels += 1;
