@@ -350,6 +350,7 @@ void amg_apply(ofks_ctx *c, const double *r_full, double *z_full);
 // ---- spmm.cu (T = double or float)
 template <class T> void launch_sell_spmm(ofks_ctx *c, const T *val, const T *X, T *Y);
 template <class T> void launch_sell_spmm_ld(ofks_ctx *c, const T *val, const T *X, T *Y, int ld);
+bool launch_spmm_masked_add(ofks_ctx *c, const float *val, const float *X, float *Y, const float *mask, int ld);
 template <class T> void launch_sell_spmm_colnorm(ofks_ctx *c, const T *val, const T *X, T *Y, double *colsum);
 // the PCG operator apply on a block of width w with pc real columns (w = ld, pc = p: all columns)
 template <class T>
