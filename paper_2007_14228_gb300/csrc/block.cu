@@ -1014,6 +1014,8 @@ void launch_grad_update(ofks_ctx *c, Blocks<T> &b) {
             return;
         }
     }
+    if constexpr (sizeof(T) == 8)
+        if (launch_grad_dig(c, b.HX, b.BX, G, c->d_sc + SC_KKT2)) return;
     const unsigned grid = row_grid(32, c->n);
     const int no = (32 * ld + 255) / 256;
 #define GR_(k) { cudaFuncSetAttribute(k_grad<T, k>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \

@@ -364,6 +364,11 @@ template <class T> void launch_gram2(ofks_ctx *c, const T *X, const T *A, const 
 bool launch_gram_tc(ofks_ctx *c, const float *X, const float *A, const float *B, double *part, int64_t *units);
 // grad_tc.cu: G = H X + B X C and |H X - B X Lambda0|^2 on the tensor cores (false: not supported)
 bool launch_grad_tc(ofks_ctx *c, const float *HX, const float *BX, float *G, double *kkt2);
+// float64 gradient by digit products on the tensor cores (grad_dig.cu), GRAD_DIG_MIN <= ld <= 48: below,
+// the direct form's 2 ld multiply-adds per entry cost no more than the digits; above, the digits of a
+// tile, of C and of Lambda0 do not fit in shared memory
+constexpr int GRAD_DIG_MIN = 16;
+bool launch_grad_dig(ofks_ctx *c, const double *HX, const double *BX, double *G, double *kkt2);
 template <class T> void launch_grad_update(ofks_ctx *c, Blocks<T> &b);
 // The PCG's working set: its block width w (row pitch of R, Z, P, Q, W and of the D it builds,
 // and the stride of its per-column arrays cb) and its real column count pc.  In the compact
