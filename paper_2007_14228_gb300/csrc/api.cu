@@ -257,11 +257,16 @@ static int download_block(ofks_ctx *c, const double *d, double *h) {
     return ofks_cuda_check(c, e, "block download");
 }
 
+// the status of the last p x p kernel; also fails where a Gram's bounded wait gave up before it
 static int read_flag(ofks_ctx *c, int *h) {
-    cudaError_t e = cudaMemcpyAsync(h, c->d_flag, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+    int f[3] = {0, 0, 0}, rc;
+    cudaError_t e = cudaMemcpyAsync(f, c->d_flag, sizeof(f), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->d_flag, 0, sizeof(int), c->stream);
-    return ofks_cuda_check(c, e, "status flag");
+    if (e == cudaSuccess && f[2]) e = cudaMemsetAsync(c->d_flag + 2, 0, sizeof(int), c->stream);
+    if ((rc = ofks_cuda_check(c, e, "status flag"))) return rc;
+    *h = f[0];
+    return f[2] ? ofks_fail(c, OFKS_ETIMEOUT, "tensor-core Gram: a bounded wait timed out") : OFKS_OK;
 }
 
 // ------------------------------------------------------------------------------ iteration

@@ -953,6 +953,14 @@ void launch_gram2(ofks_ctx *c, const T *X, const T *A, const T *B, double *XA, d
             return;
         }
     }
+    if constexpr (sizeof(T) == 8) {
+        int ts = 0, nt = 0;
+        int64_t units = 0;
+        if (launch_gram_dig(c, X, A, B, c->d_cpart, &ts, &nt, &units)) {
+            fin(ts, nt, units);
+            return;
+        }
+    }
     int RT = p <= 16 ? 1 : (p <= 32 ? 2 : (p <= 48 ? 3 : 4));
     const int TS = 16 * RT, ntile = (p + TS - 1) / TS, npair = ntile * (ntile + 1) / 2;
     int64_t splits = std::max<int64_t>(1, std::min<int64_t>((c->n + 255) / 256, (152LL * 4) / npair + 1));

@@ -41,30 +41,55 @@ __device__ __forceinline__ void split(double v, int e, uint32_t (&q)[ND]) {
     }
 }
 
-// (hi 2^27 + lo) 2^e rounded to float64 (to nearest, ties away from zero; subnormal results are zero)
+// (hi 2^SH + lo) 2^e rounded to float64 (to nearest, ties away from zero; subnormal results are zero)
+template <int SH>
 __device__ __forceinline__ double combine(long long hi, long long lo, int e) {
-    long long H = hi + (lo >> 27);
-    uint32_t rem = (uint32_t)lo & 0x7ffffffu;
+    constexpr uint32_t LOW = SH == 32 ? 0xffffffffu : (1u << (SH & 31)) - 1u;
+    long long H = hi + (lo >> SH);
+    uint32_t rem = (uint32_t)lo & LOW;
     const bool neg = H < 0;
     if (neg) {
         H = -H - (rem ? 1 : 0);
-        rem = (0x8000000u - rem) & 0x7ffffffu;
+        rem = (0u - rem) & LOW;
     }
     if (H == 0) {
         if (rem == 0) return 0.0;
         H = rem;
         rem = 0;
-        e -= 27;
+        e -= SH;
     }
     const int lz = __clzll(H);
     const unsigned long long M =
-        ((unsigned long long)H << lz) | (lz >= 27 ? (unsigned long long)rem << (lz - 27) : (unsigned long long)rem >> (27 - lz));
+        ((unsigned long long)H << lz) | (lz >= SH ? (unsigned long long)rem << (lz - SH) : (unsigned long long)rem >> (SH - lz));
     const unsigned long long mant = (M >> 11) + ((M >> 10) & 1);
-    const int ex = 38 - lz + e + 52 + 1023;
+    const int ex = 63 - lz + SH + e + 1023;
     unsigned long long bits = ((unsigned long long)ex << 52) + (mant - 0x10000000000000ull);
     if (ex <= 0) bits = 0;
     if (ex >= 2046) bits = 0x7ff0000000000000ull;
     return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
+}
+
+// Eight digits of eight bits, for sums over many rows (digit products are below 2^14, so 64 of them
+// in each of eight pairs stay exact; pairs with s + t > 7 are dropped, below 2^-57 of the product of the
+// two largest magnitudes per term): f = round(v 2^(1084 - e)), |f| < 2^62, f = sum_s q_s 2^(8 (7 - s)),
+// -128 <= q_s < 128.  With 128 added to every digit they are the bytes of one integer.  Byte s of the
+// result (from the top) is q_s + 128.
+constexpr int NB = 8;
+
+__device__ __forceinline__ unsigned long long bytes_of(double v, int e) {
+    const long long b = __double_as_longlong(v);
+    const int ev = (int)((b >> 52) & 0x7ff), down = e - ev - 9;
+    long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
+    if (down <= 0) m <<= -down;
+    else m = down < 62 ? ((m >> (down - 1)) + 1) >> 1 : 0;
+    if (ev == 0) m = 0;                           // zeros and subnormals
+    if (b < 0) m = -m;
+    return (unsigned long long)m + 0x8080808080808080ull;
+}
+
+// byte k of w, less 128, as the bits of a float32 (its high half is the bf16)
+__device__ __forceinline__ uint32_t digit_of(uint32_t w, int k) {
+    return __float_as_uint(__uint_as_float(__byte_perm(w, 0x4b000000u, 0x7650u | (uint32_t)k)) - 8388736.f);
 }
 
 }  // namespace dig

@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(OTH, 1) k_grad_dig(int64_t n, int p, int ld, i
 #pragma unroll
                     for (int d = 4; d < dig::ND; ++d) lo = (lo << 9) + (int)v[d][j];
                     const int eC = sEC[m][col0 + cb + j];
-                    double val = dig::combine(hi, lo, eR + eC - 2 * 1083 + 54);
+                    double val = dig::combine<27>(hi, lo, eR + eC - 2 * 1083 + 54);
                     if (eR == 2047 || eC == 2047) val = __longlong_as_double(0x7ff8000000000000ll);
                     const int col = col0 + cb + j;
                     if (m == 0) g[j] = h[cb + j] + val;

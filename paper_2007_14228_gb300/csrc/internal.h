@@ -369,6 +369,11 @@ bool launch_grad_tc(ofks_ctx *c, const float *HX, const float *BX, float *G, dou
 // tile, of C and of Lambda0 do not fit in shared memory
 constexpr int GRAD_DIG_MIN = 16;
 bool launch_grad_dig(ofks_ctx *c, const double *HX, const double *BX, double *G, double *kkt2);
+// float64 Grams by digit products (gram_dig.cu), ld >= GRAM_DIG_MIN (below, the direct form's ld multiply-adds
+// per entry cost no more than the digits): partials for k_gram_fin
+constexpr int GRAM_DIG_MIN = 16;
+bool launch_gram_dig(ofks_ctx *c, const double *X, const double *A, const double *B, double *part, int *ts, int *ntile,
+                     int64_t *units);
 template <class T> void launch_grad_update(ofks_ctx *c, Blocks<T> &b);
 // The PCG's working set: its block width w (row pitch of R, Z, P, Q, W and of the D it builds,
 // and the stride of its per-column arrays cb) and its real column count pc.  In the compact
