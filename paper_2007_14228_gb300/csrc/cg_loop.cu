@@ -1,15 +1,23 @@
 // The Hartree CG with the separable preconditioner as one persistent cooperative kernel.
 //
-// A CG iteration is five dependent phases (lattice SpMV; update and forward pass; middle pass;
-// backward pass; direction), each a few microseconds of work below half a million nodes.  As
-// kernels of their own (ten launches with the six-pass preconditioner) they cost 112 us per
-// iteration at 49^3 nodes, most of it launch latency, reloading the axis matrices and draining;
-// here one CTA per SM keeps the six axis matrices, the stencil tables and its tensor memory for
-// the whole solve, the phases are separated by grid barriers, and the residual test (with the
-// iteration counts it is taken at) runs on the device, so a solve is one launch and one host
-// synchronization: 44 us per iteration at 49^3 nodes (float64 SpMV 10, forward 6, middle 4,
-// backward 6, direction 3, five barriers at 1.5 and the two scalars at 2), 92 against 190 at
-// 121x65x61 (float-float SpMV 31).  float64 operations of a warp take 16 cycles each, so the
+// As kernels of their own (ten launches with the six-pass preconditioner) an iteration's phases cost
+// 112 us at 49^3 nodes, most of it launch latency, reloading the axis matrices and draining; here
+// one CTA per SM keeps the six axis matrices, the stencil tables and its tensor memory for the whole
+// solve, the phases are separated by grid barriers, and the residual test (with the iteration
+// counts it is taken at) runs on the device, so a solve is one launch and one host synchronization.
+//
+// The iteration is Chronopoulos and Gear's arrangement of CG (J. Comput. Appl. Math. 25, 1989): the
+// operator is applied to z = A_sep^-1 r instead of p, w = L z, and s = L p follows by recurrence,
+//   beta = (r.z)' / (r.z),  alpha = r.z / (z.w - beta r.z / alpha_previous),
+//   p = z + beta p,  s = w + beta s,  U += alpha p,  r -= alpha s,
+// so both sums are known after one phase, and the four phases of an iteration are
+//   middle pass | backward pass, r.z | SpMV, z.w | update and forward pass, r.r.
+// p and U need only their own node, so CTAs without a plane of the forward pass take them (or, where
+// few are left over, all CTAs behind their middle tiles).  z has float32 values, which halves the
+// float-float SpMV's gathers.  A test that passes ends the solve before the middle pass.
+//
+// Measured against the usual arrangement (SpMV on p, five barriers), Hartree solves of four steps: 8^3
+// cells 2.46 -> 2.38 ms, 24^3 3.41 -> 3.15, 21x19x23 3.40 -> 3.20, 60x32x30 (float-float) 4.45 -> 4.01.  float64 operations of a warp take 16 cycles each, so the
 // passes that run on few SMs hold as few of them as possible.  512 threads and eight loads in
 // flight per lane measured best (256: 50 us at 49^3 and 120 at 121x65x61; 768: 49 and 102).
 //
@@ -45,10 +53,9 @@ struct Loop {
     int tcols;
     Vecs V;
     double *p;
-    float *zf;                                    // z, float32 (in the room of the float64 z)
-    float2 *pf;                                   // p as float32 pairs (float-float SpMV); null: float64
+    float *zf;                                    // z, float32 (in the room of the float64 z; float-float SpMV)
     const double *rhs;
-    double *q;
+    double *q;                                    // w = L z
     int Lx;
     const StencilType *types;
     const StencilCode *code;
@@ -56,7 +63,7 @@ struct Loop {
     const float2 *valff;
     double tol2, rate;
     int max_iter;
-    double *part;                                 // 4 x gridDim.x: pq, rr, rz, |rhs|^2
+    double *part;                                 // 4 x gridDim.x: zw, rr, rz, |rhs|^2
     CgOut *out;
 };
 
@@ -91,6 +98,18 @@ __device__ __forceinline__ double grid_total(const double *part, double *s_val) 
     return *s_val;
 }
 
+// two such sums, one by each of the first two warps
+__device__ __forceinline__ void grid_totals(const double *p0, const double *p1, double *s_two) {
+    if (threadIdx.x < 64) {
+        const double *part = threadIdx.x < 32 ? p0 : p1;
+        double s = 0.0;
+        for (unsigned i = threadIdx.x & 31; i < gridDim.x; i += 32) s += __ldcg(part + i);
+        s = warp_sum(s);
+        if ((threadIdx.x & 31) == 0) s_two[threadIdx.x >> 5] = s;
+    }
+    __syncthreads();
+}
+
 struct Tables {
     StencilType type[8];
     StencilCode code[8 * ST_MAXE];
@@ -104,15 +123,16 @@ struct Row {
 };
 
 // the row's product with x over its entries in the order of the stencil kernels, BATCH loads at a time
-template <class F2, class Get, class Acc>
-__device__ __forceinline__ void row_product(const Tables &tb, const Row &R, const F2 *__restrict__ val, Get get, Acc acc) {
+template <class F2, class X2, class Get, class Acc>
+__device__ __forceinline__ void row_product(const Tables &tb, const Row &R, const F2 *__restrict__ val, X2, Get get, Acc acc) {
     const StencilCode *se = tb.code + R.t * ST_MAXE;
-    auto fetch = [&](const StencilCode &E, F2 &v, F2 &x) {
+    auto fetch = [&](const StencilCode &E, F2 &v, X2 &x) {
         const int lo = E.lin4 & 1 ? R.idx[1] : R.idx[0], hi = E.lin4 & 1 ? R.idx[3] : R.idx[2];
         v = __ldg(val + E.off + (E.lin4 & 2 ? hi : lo));
         x = get(R.node + (E.lin4 >> 2));
     };
-    F2 v[BATCH], x[BATCH];
+    F2 v[BATCH];
+    X2 x[BATCH];
     int e = R.e0;
     for (; e + BATCH <= R.e1; e += BATCH) {
 #pragma unroll
@@ -128,11 +148,10 @@ __device__ __forceinline__ void row_product(const Tables &tb, const Row &R, cons
         if (e + u < R.e1) acc(v[u], x[u]);
 }
 
-__device__ __forceinline__ void ff_madd(float &sh, float &sl, const float2 a, const float2 x) {
-    const float p = __fmul_rn(a.x, x.x);
-    float e = __fmaf_rn(a.x, x.x, -p);
-    e = __fmaf_rn(a.x, x.y, e);
-    e = __fmaf_rn(a.y, x.x, e);
+__device__ __forceinline__ void ff_madd(float &sh, float &sl, const float2 a, const float x) {
+    const float p = __fmul_rn(a.x, x);
+    float e = __fmaf_rn(a.x, x, -p);
+    e = __fmaf_rn(a.y, x, e);
     const float t = __fadd_rn(sh, p);
     const float bv = __fsub_rn(t, sh);
     const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bv)), __fsub_rn(p, bv));
@@ -182,13 +201,13 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag, s_abort, s_chunk;
-    __shared__ double sh[NW], s_val, s_coef;
+    __shared__ double sh[NW], s_val, s_coef, s_two[2], s_ab[2];
     __shared__ float s_l[64];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned G = gridDim.x;
     const uint32_t sm = su32(dsm), sB = sm + P.oB;
     const int mtx = (P.px + 127) >> 7, mty = (P.py + 127) >> 7, mtz = (P.pz + 127) >> 7;
-    double *part_pq = P.part, *part_rr = P.part + G, *part_rz = P.part + 2 * G, *part_bb = P.part + 3 * G;
+    double *part_zw = P.part, *part_rr = P.part + G, *part_rz = P.part + 2 * G, *part_bb = P.part + 3 * G;
     for (int i = threadIdx.x; i < 8 * ST_MAXE; i += NTH) tb.code[i] = P.code[i];
     if (threadIdx.x < 8) tb.type[threadIdx.x] = P.types[threadIdx.x];
     if (threadIdx.x == 0) {
@@ -211,13 +230,13 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
         for_rows(P, tb,
                  [&](const Row &R) {
                      double s = 0.0;
-                     row_product(tb, R, P.val, [&](int j) { return P.V.U[j]; }, [&](double v, double x) { s = fma(v, x, s); });
+                     row_product(tb, R, P.val, 0.0, [&](int j) { return P.V.U[j]; }, [&](double v, double x) { s = fma(v, x, s); });
                      return s;
                  },
                  [&](const Row &R, bool in, double s) {
                      if (!in) {
                          P.V.r[R.node] = 0.0; P.p[R.node] = 0.0;
-                         if (FF) P.pf[R.node] = make_float2(0.f, 0.f);
+                         if (FF) P.zf[R.node] = 0.f; else P.V.z[R.node] = 0.0;
                          return;
                      }
                      const double f = P.rhs[R.node], ri = f - s;
@@ -236,13 +255,30 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
     double rr = grid_total(part_rr, &s_val), rr_prev = 0.0, rz = 0.0, rate = P.rate;
     int it = 0, it_prev = 0, status = OFKS_OK;
 
-    // the three passes; with update the CG update r -= alpha q first.  Leaves r.z's partials.
-    auto precondition = [&](bool update, double alpha) -> bool {
-        double none = 0.0, prz = 0.0;
+    // p = z + beta p, U += alpha p on the interior (warps over the rows along c) by CTAs c0, c0 + 1, ...
+    auto direction = [&](double alpha, double beta, int c0) {
+        const int nc = (int)G - c0;
+        if ((int)blockIdx.x < c0) return;
+        for (int row = warp * nc + (int)blockIdx.x - c0; row < P.nx * P.ny; row += NW * nc) {
+            const int a = row / P.ny, b = row - a * P.ny;
+            const int o = ((a + 1) * P.V.Ly + (b + 1)) * P.V.Lz + 1;
+            for (int cc = lane; cc < P.nz; cc += 32) {
+                double v = FF ? f2d_bits(P.zf[o + cc]) : P.V.z[o + cc];
+                if (beta != 0.0) v = fma(beta, P.p[o + cc], v);
+                P.p[o + cc] = v;
+                P.V.U[o + cc] = fma(alpha, v, P.V.U[o + cc]);
+            }
+        }
+    };
+    // forward pass; with update the CG update of s and r first, leaving r.r's partials (and p and U, where
+    // at least half of the CTAs have no plane)
+    const bool spare = (int)G >= 2 * P.nx;
+    auto forward = [&](bool update, double alpha, double beta) -> bool {
+        double prr = 0.0;
         bool good = true;
         for (int a = blockIdx.x; a < P.nx && good; a += G) {
-            if (update) residual_to_data<NW, 1, 0>(P.V, a, P.ny, P.nz, P.py, P.pz, alpha, none, dsm, P.oB, P.part_p);
-            else residual_to_data<NW, 0, 0>(P.V, a, P.ny, P.nz, P.py, P.pz, alpha, none, dsm, P.oB, P.part_p);
+            if (update) residual_to_data<NW, 2>(P.V, a, P.ny, P.nz, P.py, P.pz, alpha, beta, prr, dsm, P.oB, P.part_p);
+            else residual_to_data<NW, 0>(P.V, a, P.ny, P.nz, P.py, P.pz, 0.0, 0.0, prr, dsm, P.oB, P.part_p);
             good = contract(c, sm + P.oSt[2], sB, P.part_p, mtz, P.py, P.pz);
             if (!good) break;
             acc_to_data<NW>(c, mtz, P.py, P.pz, sB, P.part_p);
@@ -250,8 +286,18 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
             if (!good) break;
             acc_to_global<NW>(c, mty, P.pz, P.ny, P.pz, P.T + (int64_t)a * P.ny * P.pz, P.pz);
         }
+        if (update) {
+            if (spare) direction(alpha, beta, P.nx);
+            const double t = cta_sum<NW>(prr, sh);
+            if (threadIdx.x == 0) part_rr[blockIdx.x] = t;
+        }
         if (!good && threadIdx.x == 0) { s_abort = 1; atomicExch(&P.out->abort, 1); }
-        if (!grid_barrier(P.out, target, &s_abort)) return false;
+        return grid_barrier(P.out, target, &s_abort);
+    };
+    // middle and backward pass: z, r.z's partials.  With pending the last update's p and U come between them.
+    auto backward = [&](bool pending, double alpha, double beta) -> bool {
+        double prz = 0.0;
+        bool good = true;
         for (int m0 = (int)blockIdx.x * P.NT; m0 < P.ncol && good; m0 += (int)G * P.NT) {
             mid_scales(P.lyzp, m0, P.ncol, P.NT, s_l);
             global_to_data<NW>(P.T + m0, P.ncol, P.nx, P.ncol - m0, P.NT, P.px, sB, P.part_m);
@@ -262,6 +308,7 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
             if (!good) break;
             acc_to_global<NW>(c, mtx, P.NT, P.nx, P.ncol - m0, P.T + m0, P.ncol);
         }
+        if (pending) direction(alpha, beta, 0);
         if (!good && threadIdx.x == 0) { s_abort = 1; atomicExch(&P.out->abort, 1); }
         if (!grid_barrier(P.out, target, &s_abort)) return false;
         for (int a = blockIdx.x; a < P.nx && good; a += G) {
@@ -271,34 +318,16 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
             acc_to_data<NW>(c, mty, P.pz, P.py, sB, P.part_p);
             good = contract(c, sm + P.oS[2], sB, P.part_p, mtz, P.py, P.pz);
             if (!good) break;
-            acc_to_z<NW, 1>(c, mtz, P.V, a, P.ny, P.nz, P.py, P.zf, nullptr, nullptr, prz);
+            acc_to_z<NW, FF>(c, mtz, P.V, a, P.ny, P.nz, P.py, P.zf, nullptr, nullptr, prz);
         }
         const double t = cta_sum<NW>(prz, sh);
         if (threadIdx.x == 0) part_rz[blockIdx.x] = t;
         if (!good && threadIdx.x == 0) { s_abort = 1; atomicExch(&P.out->abort, 1); }
         return grid_barrier(P.out, target, &s_abort);
     };
-    // U += alpha p, p = z + beta p and r.r on the interior (warps over the rows along c), spread over
-    // the whole grid: the passes over planes run on as many CTAs as there are planes, and every
-    // float64 operation of a warp takes 16 cycles
-    auto direction = [&](double alpha, double beta) {
-        double prr = 0.0;
-        for (int row = warp * G + blockIdx.x; row < P.nx * P.ny; row += NW * G) {
-            const int a = row / P.ny, b = row - a * P.ny;
-            const int o = ((a + 1) * P.V.Ly + (b + 1)) * P.V.Lz + 1;
-            for (int cc = lane; cc < P.nz; cc += 32) {
-                const double pv = P.p[o + cc], zv = f2d_bits(P.zf[o + cc]), rv = P.V.r[o + cc];
-                if (alpha != 0.0) P.V.U[o + cc] = fma(alpha, pv, P.V.U[o + cc]);
-                const double v = beta != 0.0 ? fma(beta, pv, zv) : zv;
-                P.p[o + cc] = v;
-                if (FF) P.pf[o + cc] = ff_split(v);
-                prr = fma(rv, rv, prr);
-            }
-        }
-        prr = cta_sum<NW>(prr, sh);
-        if (threadIdx.x == 0) part_rr[blockIdx.x] = prr;
-    };
 
+    double alpha = 0.0, beta = 0.0;
+    bool pending = false;
     while (ok) {
         // the residual test, and the iterations to the next one: the count that the last observed
         // factor of the squared residual predicts to the target, 1 to 8 (4 before any is known)
@@ -326,25 +355,20 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
         rate = s_coef;
         rr_prev = rr;
         it_prev = it;
-        if (it == 0) {                            // z = A_sep^-1 r, p = z
-            ok = precondition(false, 0.0);
-            if (!ok) break;
-            rz = grid_total(part_rz, &s_val);
-            direction(0.0, 0.0);
-            ok = grid_barrier(P.out, target, &s_abort);
-        }
+        if (it == 0) ok = forward(false, 0.0, 0.0);
         for (int j = 0; j < chunk && ok; ++j) {
-            double pq = 0.0;
+            if (!(ok = backward(pending, alpha, beta))) break;
+            double zw = 0.0;
             for_rows(P, tb,
                      [&](const Row &R) {
                          if constexpr (FF) {
                              float s_hi = 0.f, s_lo = 0.f;
-                             row_product(tb, R, P.valff, [&](int i) { return P.pf[i]; },
-                                         [&](float2 v, float2 x) { ff_madd(s_hi, s_lo, v, x); });
+                             row_product(tb, R, P.valff, 0.f, [&](int i) { return P.zf[i]; },
+                                         [&](float2 v, float x) { ff_madd(s_hi, s_lo, v, x); });
                              return (double)s_hi + (double)s_lo;
                          } else {
                              double s = 0.0;
-                             row_product(tb, R, P.val, [&](int i) { return P.p[i]; },
+                             row_product(tb, R, P.val, 0.0, [&](int i) { return P.V.z[i]; },
                                          [&](double v, double x) { s = fma(v, x, s); });
                              return s;
                          }
@@ -352,28 +376,30 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
                      [&](const Row &R, bool in, double s) {
                          if (!in) return;
                          P.q[R.node] = s;
-                         pq = fma(P.p[R.node], s, pq);
+                         zw = fma(FF ? f2d_bits(P.zf[R.node]) : P.V.z[R.node], s, zw);
                      });
-            const double tpq = cta_sum<NW>(pq, sh);
-            if (threadIdx.x == 0) part_pq[blockIdx.x] = tpq;
+            const double tzw = cta_sum<NW>(zw, sh);
+            if (threadIdx.x == 0) part_zw[blockIdx.x] = tzw;
             if (!(ok = grid_barrier(P.out, target, &s_abort))) break;
-            const double den = grid_total(part_pq, &s_val);
-            if (threadIdx.x == 0) s_coef = den > 0.0 ? rz / den : 0.0;
+            grid_totals(part_rz, part_zw, s_two);
+            if (threadIdx.x == 0) {
+                const double b = it > 0 && rz > 0.0 ? s_two[0] / rz : 0.0;
+                const double den = alpha != 0.0 ? s_two[1] - b * s_two[0] / alpha : s_two[1];
+                s_ab[0] = den > 0.0 ? s_two[0] / den : 0.0;
+                s_ab[1] = b;
+            }
             __syncthreads();
-            const double alpha = s_coef;
-            if (!(ok = precondition(true, alpha))) break;
-            const double rz2 = grid_total(part_rz, &s_val);
-            if (threadIdx.x == 0) s_coef = rz > 0.0 ? rz2 / rz : 0.0;
-            __syncthreads();
-            const double beta = s_coef;
-            rz = rz2;
-            direction(alpha, beta);
-            ok = grid_barrier(P.out, target, &s_abort);
+            rz = s_two[0];
+            alpha = s_ab[0];
+            beta = s_ab[1];
+            ok = forward(true, alpha, beta);
+            pending = !spare;
             ++it;
         }
         if (ok) rr = grid_total(part_rr, &s_val);
         __syncthreads();
     }
+    if (ok && pending) direction(alpha, beta, 0);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         P.out->rr = rr; P.out->bb = bb; P.out->rate = rate; P.out->it = it; P.out->status = status;
     }
@@ -421,8 +447,8 @@ int cg_loop_run(ofks_ctx *c, double tol2, int *iters, int *status, double *rel2)
     SepState &S = c->sep;
     Loop P{};
     const int smem = place_loop(S, P);
-    P.V = {c->st.Ly, c->st.Lz, c->d_cp, c->d_cq, c->d_U, c->d_cr, c->d_cz};
-    P.p = c->d_cp; P.zf = reinterpret_cast<float *>(c->d_cz); P.q = c->d_cq; P.pf = c->hartree_ff ? c->d_cpff : nullptr; P.rhs = c->d_rhs;
+    P.V = {c->st.Ly, c->st.Lz, c->d_cp, c->d_cq, c->d_U, c->d_cr, c->d_cz, reinterpret_cast<double *>(c->d_cpff)};
+    P.p = c->d_cp; P.zf = reinterpret_cast<float *>(c->d_cz); P.q = c->d_cq; P.rhs = c->d_rhs;
     P.Lx = c->st.Lx;
     P.types = c->st.d_type; P.code = c->st.d_code; P.val = c->st.val; P.valff = c->st.valff;
     P.tol2 = tol2; P.rate = c->cg_rate; P.max_iter = c->prm.poisson_max_iter;

@@ -56,8 +56,8 @@ __global__ void __launch_bounds__(NT_, 2) k_plane_fwd(const Plane P) {
     Cta c;
     cta_open(c, &mbar, &tmem_base, &abort_flag, P.tcols);
     double rr = 0.0;
-    if (P.it >= 0) residual_to_data<NW_, 1, 1>(P.V, a, P.ny, P.nz, P.py, P.pz, s_alpha, rr, dsm, P.oB, P.part);
-    else residual_to_data<NW_, 0, 0>(P.V, a, P.ny, P.nz, P.py, P.pz, 0.0, rr, dsm, P.oB, P.part);
+    if (P.it >= 0) residual_to_data<NW_, 1>(P.V, a, P.ny, P.nz, P.py, P.pz, s_alpha, 0.0, rr, dsm, P.oB, P.part);
+    else residual_to_data<NW_, 0>(P.V, a, P.ny, P.nz, P.py, P.pz, 0.0, 0.0, rr, dsm, P.oB, P.part);
     if (contract(c, sm, sB, P.part, mtz, P.py, P.pz)) {
         if (P.late) load_axis<NW_>(sm, P.Sb, P.py);
         acc_to_data<NW_>(c, mtz, P.py, P.pz, sB, P.part);          // row k, columns b
@@ -191,7 +191,7 @@ void sep_plane_hartree(ofks_ctx *c, int it, int slot, int first) {
     Plane P;
     Middle M;
     auto vectors = [&]() {
-        P.V = {c->st.Ly, c->st.Lz, c->d_cp, c->d_cq, c->d_U, c->d_cr, c->d_cz};
+        P.V = {c->st.Ly, c->st.Lz, c->d_cp, c->d_cq, c->d_U, c->d_cr, c->d_cz, nullptr};
         P.pw = first ? c->d_cp : nullptr; P.pf = first && c->hartree_ff ? c->d_cpff : nullptr;
         P.sc = c->d_sc + SC_CG; P.it = it; P.slot = slot; P.gpart = c->d_gpart; P.gcount = c->d_gcount;
     };

@@ -277,17 +277,20 @@ struct Vecs {
     int Ly, Lz;
     const double *p, *q;
     double *U, *r, *z;
+    double *s;
 };
 
-// plane a of the residual -> data operand (n = b, k = c), zero outside the interior.  With UPDATE the
-// CG update r -= alpha q comes first, and with FULL also U += alpha p and rr += r.r.
-template <int NW, int UPDATE, int FULL>
-__device__ __forceinline__ void residual_to_data(const Vecs &V, int a, int ny, int nz, int py, int pz, double alpha,
+// plane a of the residual -> data operand (n = b, k = c), zero outside the interior.  With UPDATE 1 the
+// CG update r -= alpha q, U += alpha p, rr += r.r comes first, with UPDATE 2 that of the single-reduction
+// form (cg_loop.cu), s = q + beta s, r -= alpha s, rr += r.r.
+template <int NW, int UPDATE>
+__device__ __forceinline__ void residual_to_data(const Vecs &V, int a, int ny, int nz, int py, int pz, double alpha, double beta,
                                                  double &rr, unsigned char *dsm, uint32_t off, uint32_t part) {
-    constexpr int PIECES = FULL ? 4 : 6;          // pieces of 32 values whose loads are issued together
+    constexpr int FULL = UPDATE == 1;
+    constexpr int PIECES = UPDATE ? 4 : 6;         // pieces of 32 values whose loads are issued together
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k8 = pz >> 3, nch = (pz + 31) >> 5;
     for (int e0 = warp; e0 < py * nch; e0 += NW * PIECES) {
-        double rv[PIECES], pv[PIECES], qv[PIECES], uv[PIECES];
+        double rv[PIECES], pv[PIECES], qv[PIECES], uv[PIECES], sv[PIECES];
         int bb[PIECES], cc[PIECES];
         int64_t at[PIECES];
         bool in[PIECES];
@@ -300,6 +303,7 @@ __device__ __forceinline__ void residual_to_data(const Vecs &V, int a, int ny, i
             at[u] = ((int64_t)(a + 1) * V.Ly + (bb[u] + 1)) * V.Lz + 1 + cc[u];
             rv[u] = in[u] ? V.r[at[u]] : 0.0;
             if (UPDATE) qv[u] = in[u] ? V.q[at[u]] : 0.0;
+            if (UPDATE == 2) sv[u] = in[u] && beta != 0.0 ? V.s[at[u]] : 0.0;
             if (FULL) pv[u] = in[u] ? V.p[at[u]] : 0.0;
             if (FULL) uv[u] = in[u] ? V.U[at[u]] : 0.0;
         }
@@ -309,9 +313,13 @@ __device__ __forceinline__ void residual_to_data(const Vecs &V, int a, int ny, i
             double ri = rv[u];
             if (UPDATE && in[u]) {
                 if (FULL) V.U[at[u]] = fma(alpha, pv[u], uv[u]);
+                if (UPDATE == 2) {
+                    if (beta != 0.0) qv[u] = fma(beta, sv[u], qv[u]);
+                    V.s[at[u]] = qv[u];
+                }
                 ri = fma(-alpha, qv[u], ri);
                 V.r[at[u]] = ri;
-                if (FULL) rr = fma(ri, ri, rr);
+                rr = fma(ri, ri, rr);
             }
             const float f = d2f_bits(ri);
             const bf hi = __float2bfloat16(f);
