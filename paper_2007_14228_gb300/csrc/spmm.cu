@@ -75,8 +75,9 @@ inline int spw_for(int64_t units) {
 // written (float64) to part[c * nsg + g] for slice group g (nsg groups of spw slices), to be
 // added in group order (launch_col_fin).  T is the element type of the values and blocks; sums
 // run in T.
-template <class T, int W, int MODE>
-__global__ void __launch_bounds__(256) k_sell_spmm(int64_t nwarps, int nchunks, int64_t n_slices, int spw_, int p, int ld,
+// Of the chunk's W columns the first R are multiplied; the others are the block's padding (zeros).
+template <class T, int W, int MODE, int R>
+__device__ __forceinline__ void sell_spmm_chunk(int64_t nwarps, int nchunks, int64_t n_slices, int spw_, int p, int ld,
                                                    const int *__restrict__ slice_ptr,
                                                    const int *__restrict__ slice_w,
                                                    const int *__restrict__ cols,
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(256) k_sell_spmm(int64_t nwarps, int nchunks, 
             T x[W];
             load_w<T, W>(X + (int64_t)c * ld + c0, x);
 #pragma unroll
-            for (int w = 0; w < W; ++w) acc[w] = fma(v, x[w], acc[w]);
+            for (int w = 0; w < R; ++w) acc[w] = fma(v, x[w], acc[w]);
         }
         if (r >= 0) {
             store_w<T, W>(Y + (int64_t)r * ld + c0, acc);
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(256) k_sell_spmm(int64_t nwarps, int nchunks, 
                 T xr[W];
                 load_w<T, W>(X + (int64_t)r * ld + c0, xr);
 #pragma unroll
-                for (int w = 0; w < W; ++w) cs[w] = fma(xr[w], acc[w], cs[w]);
+                for (int w = 0; w < R; ++w) cs[w] = fma(xr[w], acc[w], cs[w]);
             }
         }
     }
@@ -130,13 +131,36 @@ __global__ void __launch_bounds__(256) k_sell_spmm(int64_t nwarps, int nchunks, 
     }
 }
 
+// float64: a multiply-add of a warp takes its pipe 16 cycles, so the last chunk leaves out the padding
+// columns (41 columns in a pitch of 44: 7 % of the multiply-adds).  PCG apply at n = 1.18 M 4.09 -> 3.76 ms, at 68k
+// 0.104 -> 0.084; H X and B Y at 1.18 M, p = 41 2.4 -> 2.2 ms
+template <class T, int W, int MODE>
+__global__ void __launch_bounds__(256) k_sell_spmm(int64_t nwarps, int nchunks, int64_t n_slices, int spw_, int p, int ld,
+                                                   const int *__restrict__ slice_ptr,
+                                                   const int *__restrict__ slice_w,
+                                                   const int *__restrict__ cols,
+                                                   const int *__restrict__ perm,
+                                                   const T *__restrict__ val,
+                                                   const T *__restrict__ X, T *__restrict__ Y,
+                                                   double *part) {
+#define R_(r) sell_spmm_chunk<T, W, MODE, r>(nwarps, nchunks, n_slices, spw_, p, ld, slice_ptr, slice_w, cols, perm, val, X, Y, part)
+    if constexpr (sizeof(T) == 8 && W == 4) {
+        const int64_t wg = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+        const int real = p - (int)(wg % nchunks) * W;           // the same for the whole warp
+        if (real >= 4) R_(4); else if (real == 3) R_(3); else if (real == 2) R_(2); else R_(1);
+    } else {
+        R_(W);
+    }
+#undef R_
+}
+
 // One Jacobi-PCG operator apply for all columns at once (Eq. precondition-T):
 //   TZ = (L/2) Z - B Z diag(shift)  gathered over the neighbours of each row, then for the
 //   own row  P <- Z + beta P,  Q <- TZ + beta Q  (so T P = Q), and the column sums P.Q of the
 // warp's slices to part[c * nsg + g] (slice group g; added in group order by k_pcg_alpha).
-// With first = 1: P = Z, Q = TZ.
-template <class T, int W>
-__global__ void __launch_bounds__(256) k_pcg_apply(int64_t nwarps, int nchunks, int64_t n_slices, int spw, int p, int ld,
+// With first = 1: P = Z, Q = TZ.  Of the chunk's W columns the first R are real (as in k_sell_spmm).
+template <class T, int W, int R>
+__device__ __forceinline__ void pcg_apply_chunk(int64_t nwarps, int nchunks, int64_t n_slices, int spw, int p, int ld,
                                                    const int *__restrict__ slice_ptr,
                                                    const int *__restrict__ slice_w,
                                                    const int *__restrict__ cols,
@@ -174,7 +198,7 @@ __global__ void __launch_bounds__(256) k_pcg_apply(int64_t nwarps, int nchunks, 
             T x[W];
             load_w<T, W>(Z + (int64_t)c * ld + c0, x);
 #pragma unroll
-            for (int w = 0; w < W; ++w) { aL[w] = fma(vl, x[w], aL[w]); aB[w] = fma(vb, x[w], aB[w]); }
+            for (int w = 0; w < R; ++w) { aL[w] = fma(vl, x[w], aL[w]); aB[w] = fma(vb, x[w], aB[w]); }
         }
         if (r >= 0) {
             T zr[W], pr[W], qr[W];
@@ -201,6 +225,30 @@ __global__ void __launch_bounds__(256) k_pcg_apply(int64_t nwarps, int nchunks, 
         const T t = warp_sum_t(contrib[w]);
         if (lane == 0) part[(int64_t)(c0 + w) * nsg + g] = (double)t;
     }
+}
+
+template <class T, int W>
+__global__ void __launch_bounds__(256) k_pcg_apply(int64_t nwarps, int nchunks, int64_t n_slices, int spw, int p, int ld,
+                                                   const int *__restrict__ slice_ptr,
+                                                   const int *__restrict__ slice_w,
+                                                   const int *__restrict__ cols,
+                                                   const int *__restrict__ perm,
+                                                   const T *__restrict__ valL,
+                                                   const T *__restrict__ valB,
+                                                   const T *__restrict__ Z, T *P, T *Q,
+                                                   const double *__restrict__ beta_col,
+                                                   const double *__restrict__ shift, double *part,
+                                                   int first) {
+#define R_(r) pcg_apply_chunk<T, W, r>(nwarps, nchunks, n_slices, spw, p, ld, slice_ptr, slice_w, cols, perm, valL, valB, Z, P, Q, \
+                                       beta_col, shift, part, first)
+    if constexpr (sizeof(T) == 8 && W == 4) {
+        const int64_t wg = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+        const int real = p - (int)(wg % nchunks) * W;
+        if (real >= 4) R_(4); else if (real == 3) R_(3); else if (real == 2) R_(2); else R_(1);
+    } else {
+        R_(W);
+    }
+#undef R_
 }
 
 // The float32 PCG apply on the type-grouped SELL with every PCG block chunk-major: element
