@@ -501,16 +501,19 @@ static int precondition_t(ofks_ctx *c) {
         const PcgView<T> &v = L.v;
         const int w = v.w;
         for (int it = L.it0; it < L.it1; ++it) {
+            // chunk-major blocks, a fixed count of iterations: D += alpha P rides in the next apply
+            const bool ride = !L.exact && pcg_zc<T>(c, w);
             {
                 ProfScope ps(c, PF_PCG_SPMM);
                 launch_pcg_apply(c, vals_L<T>(c), vals_B<T>(c), (const T *)b.Z, pcg_zc<T>(c, w) ? 1 : 0, b.P, b.Q,
-                                 v.cb + CB_BETA * w, v.cb + CB_SHIFT * w, v.cb + CB_PQ * w, it == 0 ? 1 : 0, w, v.pc);
+                                 v.cb + CB_BETA * w, v.cb + CB_SHIFT * w, v.cb + CB_PQ * w, it == 0 ? 1 : 0, w, v.pc,
+                                 ride ? v.D : (T *)nullptr, v.cb + CB_ALPHA * w);
             }
             const bool last = !L.exact && it + 1 == L.max_it;
             {
                 ProfScope ps(c, PF_PCG_UPDATE);
                 launch_pcg_alpha(c, w, v.pc, v.cb);
-                launch_pcg_update(c, b, v, last);
+                launch_pcg_update(c, b, v, last, ride);
             }
             if (!last && c->prm.pcg_pc == OFKS_PCGPC_SEPARABLE) {
                 ProfScope ps(c, PF_PCG_SEP);

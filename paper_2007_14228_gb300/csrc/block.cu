@@ -630,11 +630,12 @@ __global__ void __launch_bounds__(256) k_pcg_init_s(int64_t n, int64_t ns, int p
 }
 
 // alpha = rz/pq; D += alpha P; R -= alpha Q; Z = R W; rzn += R Z, per float4 of one row and
-// chunk.  On the last iteration only D is needed (last = 1: R, Z and rzn are left alone).
+// chunk.  On the last iteration only D is needed (last = 1: R, Z and rzn are left alone); on the
+// others D is left to the next apply with ride = 1.
 __global__ void __launch_bounds__(256) k_pcg_update_s(int64_t ns, int pc, int w, const double *__restrict__ cb,
                                                       const float *__restrict__ W, const float *__restrict__ P,
                                                       const float *__restrict__ Q, float *D, float *R, float *Z,
-                                                      double *part, int last, int jac) {
+                                                      double *part, int last, int jac, int ride) {
     __shared__ float csw[8][MAXLD], al[MAXLD];
     for (int k = threadIdx.x; k < 8 * MAXLD; k += blockDim.x) csw[k / MAXLD][k % MAXLD] = 0.f;
     for (int k = threadIdx.x; k < w; k += blockDim.x) al[k] = (float)cb[CB_ALPHA * w + k];
@@ -646,10 +647,12 @@ __global__ void __launch_bounds__(256) k_pcg_update_s(int64_t ns, int pc, int w,
         const int q = (int)(idx / ns);
         const int64_t o = idx << 2;                  // sidx(r, 4 q, ns) with r = idx - q ns
         const float a0 = al[4 * q], a1 = al[4 * q + 1], a2 = al[4 * q + 2], a3 = al[4 * q + 3];
-        const float4 p4 = *reinterpret_cast<const float4 *>(P + o);
-        float4 d4 = *reinterpret_cast<const float4 *>(D + o);
-        d4.x = fmaf(a0, p4.x, d4.x); d4.y = fmaf(a1, p4.y, d4.y); d4.z = fmaf(a2, p4.z, d4.z); d4.w = fmaf(a3, p4.w, d4.w);
-        *reinterpret_cast<float4 *>(D + o) = d4;
+        if (last || !ride) {
+            const float4 p4 = *reinterpret_cast<const float4 *>(P + o);
+            float4 d4 = *reinterpret_cast<const float4 *>(D + o);
+            d4.x = fmaf(a0, p4.x, d4.x); d4.y = fmaf(a1, p4.y, d4.y); d4.z = fmaf(a2, p4.z, d4.z); d4.w = fmaf(a3, p4.w, d4.w);
+            *reinterpret_cast<float4 *>(D + o) = d4;
+        }
         if (last) continue;
         const float4 q4 = *reinterpret_cast<const float4 *>(Q + o);
         float4 r4 = *reinterpret_cast<const float4 *>(R + o);
@@ -1122,7 +1125,7 @@ void launch_judge(ofks_ctx *c, Blocks<T> &b) {
 }
 
 template <class T>
-void launch_pcg_update(ofks_ctx *c, Blocks<T> &b, const PcgView<T> &v, bool last) {
+void launch_pcg_update(ofks_ctx *c, Blocks<T> &b, const PcgView<T> &v, bool last, bool ride) {
     c->kernels += 1;
     const int w = v.w;
     double *cb = v.cb;
@@ -1133,7 +1136,7 @@ void launch_pcg_update(ofks_ctx *c, Blocks<T> &b, const PcgView<T> &v, bool last
             const unsigned grid = (unsigned)std::min<int64_t>((total + 255) / 256, 152 * 8);
             k_pcg_update_s<<<grid, 256, 0, c->stream>>>(
                 c->n_slots, v.pc, w, cb, (const float *)b.W, (const float *)b.P, (const float *)b.Q, (float *)v.D,
-                (float *)b.R, (float *)b.Z, c->d_cpart, last ? 1 : 0, pcg_sep_active(c, w) ? 0 : 1);
+                (float *)b.R, (float *)b.Z, c->d_cpart, last ? 1 : 0, pcg_sep_active(c, w) ? 0 : 1, ride ? 1 : 0);
             c->rz_units = grid;
             return;
         }
@@ -1272,7 +1275,7 @@ void launch_convert(ofks_ctx *c, const S *src, T *dst, int64_t count) {
     template void launch_gram2<T>(ofks_ctx *, const T *, const T *, const T *, double *, double *); \
     template void launch_grad_update<T>(ofks_ctx *, Blocks<T> &);                                    \
     template void launch_pcg_init<T>(ofks_ctx *, Blocks<T> &, const PcgView<T> &, bool);             \
-    template void launch_pcg_update<T>(ofks_ctx *, Blocks<T> &, const PcgView<T> &, bool);           \
+    template void launch_pcg_update<T>(ofks_ctx *, Blocks<T> &, const PcgView<T> &, bool, bool);     \
     template void launch_direction_expand<T>(ofks_ctx *, Blocks<T> &, const PcgView<T> &);           \
     template void launch_judge<T>(ofks_ctx *, Blocks<T> &);                                          \
     template bool launch_pcg_sep<T>(ofks_ctx *, Blocks<T> &, const PcgView<T> &);                    \

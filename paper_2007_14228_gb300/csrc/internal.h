@@ -352,10 +352,12 @@ template <class T> void launch_sell_spmm(ofks_ctx *c, const T *val, const T *X, 
 template <class T> void launch_sell_spmm_ld(ofks_ctx *c, const T *val, const T *X, T *Y, int ld);
 bool launch_spmm_masked_add(ofks_ctx *c, const float *val, const float *X, float *Y, const float *mask, int ld);
 template <class T> void launch_sell_spmm_colnorm(ofks_ctx *c, const T *val, const T *X, T *Y, double *colsum);
-// the PCG operator apply on a block of width w with pc real columns (w = ld, pc = p: all columns)
+// the PCG operator apply on a block of width w with pc real columns (w = ld, pc = p: all columns);
+// chunk-major blocks (zc): with Dlast also D += alpha_col P of the iteration before, unless first
 template <class T>
 void launch_pcg_apply(ofks_ctx *c, const T *valL, const T *valB, const T *Zin, int zc, T *P, T *Q, const double *beta_col,
-                      const double *shift, double *pq, int first, int w, int pc);
+                      const double *shift, double *pq, int first, int w, int pc, T *Dlast = nullptr,
+                      const double *alpha_col = nullptr);
 
 // ---- block.cu (tall-skinny products and vector updates)
 template <class T> void launch_gram2(ofks_ctx *c, const T *X, const T *A, const T *B, double *XA, double *XB);
@@ -393,8 +395,8 @@ template <class T> bool pcg_zc(const ofks_ctx *c, int w);
 // warm: the columns flagged in the view's CB_WARM row start from the natural-layout D (with
 // T D in Q) instead of zero
 template <class T> void launch_pcg_init(ofks_ctx *c, Blocks<T> &b, const PcgView<T> &v, bool warm = false);
-// last: the final iteration, after which only D is read
-template <class T> void launch_pcg_update(ofks_ctx *c, Blocks<T> &b, const PcgView<T> &v, bool last);
+// last: the final iteration, after which only D is read; ride: before it the next apply adds alpha P to D
+template <class T> void launch_pcg_update(ofks_ctx *c, Blocks<T> &b, const PcgView<T> &v, bool last, bool ride);
 template <class T> void launch_judge(ofks_ctx *c, Blocks<T> &b);
 // Z = T_sep^-1 R (separable preconditioner of the PCG, float32 chunk-major blocks on lattice
 // meshes) with the rz partials; false when that form does not apply

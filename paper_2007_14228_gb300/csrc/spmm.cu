@@ -251,19 +251,31 @@ __global__ void __launch_bounds__(256) k_pcg_apply(int64_t nwarps, int nchunks, 
 #undef R_
 }
 
+constexpr int ZC_U = 7;                           // entries per pass of k_pcg_apply_zc
+
 // The float32 PCG apply on the type-grouped SELL with every PCG block chunk-major: element
 // (r, c) at ((c / 4) ns + r) 4 + c % 4 (ns = n rounded up to 32), rows in type order.  A warp
 // takes spw consecutive slices in turn for one 4-column chunk and writes its column sums P.Q once
 // at the end.  Its lanes are 32 consecutive rows of one lattice node type, so for one entry index
 // their neighbours are (mostly) 32 consecutive rows of one type: each 16-byte gather of the warp
-// reads 512 contiguous bytes, and the lanes' own P and Q pieces are contiguous too.
-__global__ void __launch_bounds__(256, 4) k_pcg_apply_zc(int64_t nwarps, int nchunks, int64_t n_slices, int spw, int p,
+// reads 512 contiguous bytes, and the lanes' own P and Q pieces are contiguous too.  With D the last
+// iteration's D += alpha P comes along: the old P is read here anyway, and the gathers leave DRAM
+// bandwidth over, which the update pass does not (update 2.76 -> 2.42 ms in 32 iterations at n = 442k,
+// p = 41, 9.4 -> 7.4 in 16 at n = 493k, p = 210).
+//
+// What bounds it: L1 and L2 under the gathers.  ZC_U of them are in flight per lane at three CTAs per
+// SM, with the next pass's column ids and values behind them: 0.191 ms per launch at n = 442k with D
+// against 0.198 without D for four gathers, the rest of a row one by one, and four CTAs.  Four gathers
+// in this form at four CTAs 0.193, at three 0.236; two chunks per warp (an id and value pair for two
+// gathers, 80 or 118 registers) 0.188 to 0.214.
+__global__ void __launch_bounds__(256, 3) k_pcg_apply_zc(int64_t nwarps, int nchunks, int64_t n_slices, int spw,
                                                       int64_t n, int64_t ns, const int *__restrict__ slice_ptr,
                                                       const int *__restrict__ slice_w,
                                                       const int *__restrict__ cols,
                                                       const float *__restrict__ valL,
                                                       const float *__restrict__ valB,
-                                                      const float *__restrict__ Zc, float *P, float *Q,
+                                                      const float *__restrict__ Zc, float *P, float *Q, float *D,
+                                                      const double *__restrict__ alpha_col,
                                                       const double *__restrict__ beta_col,
                                                       const double *__restrict__ shift, double *part, int first) {
     const int64_t wg = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -276,45 +288,41 @@ __global__ void __launch_bounds__(256, 4) k_pcg_apply_zc(int64_t nwarps, int nch
     const int64_t cbase = (int64_t)chunk * ns * 4;
     const float *Zk = Zc + cbase;
     float *Pk = P + cbase, *Qk = Q + cbase;
-    float sh[4], bt[4];
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        sh[w] = (float)shift[c0 + w];
-        bt[w] = first ? 0.f : (float)beta_col[c0 + w];
-    }
     float contrib[4] = {0.f, 0.f, 0.f, 0.f};
     for (int64_t s = s0; s < s1; ++s) {
         const int base = slice_ptr[s], width = slice_w[s];
         const int64_t r = s * SELL_C + lane;
         float aL[4] = {0.f, 0.f, 0.f, 0.f}, aB[4] = {0.f, 0.f, 0.f, 0.f};
-        // four entries per pass with all their loads issued before the first multiply-add: four
-        // gathers in flight per lane (with the register cap of four CTAs per SM this measured
-        // 0.195 ms per launch against 0.34 ms for one entry per pass on the 60x32x30 chain)
-        int e = base + lane, j = 0;
-        for (; j + 4 <= width; j += 4, e += 4 * SELL_C) {
-            int cc[4];
-            float vl[4], vb[4];
-            float4 x[4];
+        int cc[ZC_U];
+        float vl[ZC_U], vb[ZC_U];
+        // past the row's end a pass repeats its last column with values of zero
+        auto entries = [&](int j) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) cc[u] = __ldg(cols + e + u * SELL_C);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) { vl[u] = __ldg(valL + e + u * SELL_C); vb[u] = __ldg(valB + e + u * SELL_C); }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = __ldg(reinterpret_cast<const float4 *>(Zk + (int64_t)cc[u] * 4));
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                aL[0] = fmaf(vl[u], x[u].x, aL[0]); aL[1] = fmaf(vl[u], x[u].y, aL[1]);
-                aL[2] = fmaf(vl[u], x[u].z, aL[2]); aL[3] = fmaf(vl[u], x[u].w, aL[3]);
-                aB[0] = fmaf(vb[u], x[u].x, aB[0]); aB[1] = fmaf(vb[u], x[u].y, aB[1]);
-                aB[2] = fmaf(vb[u], x[u].z, aB[2]); aB[3] = fmaf(vb[u], x[u].w, aB[3]);
+            for (int u = 0; u < ZC_U; ++u) {
+                const bool in = j + u < width;
+                const int e = base + lane + (in ? j + u : width - 1) * SELL_C;
+                cc[u] = __ldg(cols + e);
+                vl[u] = in ? __ldg(valL + e) : 0.f;
+                vb[u] = in ? __ldg(valB + e) : 0.f;
             }
-        }
-        for (; j < width; ++j, e += SELL_C) {
-            const int c = __ldg(cols + e);
-            const float vl = __ldg(valL + e), vb = __ldg(valB + e);
-            const float4 x = __ldg(reinterpret_cast<const float4 *>(Zk + (int64_t)c * 4));
-            aL[0] = fmaf(vl, x.x, aL[0]); aL[1] = fmaf(vl, x.y, aL[1]); aL[2] = fmaf(vl, x.z, aL[2]); aL[3] = fmaf(vl, x.w, aL[3]);
-            aB[0] = fmaf(vb, x.x, aB[0]); aB[1] = fmaf(vb, x.y, aB[1]); aB[2] = fmaf(vb, x.z, aB[2]); aB[3] = fmaf(vb, x.w, aB[3]);
+        };
+        if (width > 0) entries(0);
+        for (int j = 0; j < width; j += ZC_U) {
+            float4 x[ZC_U];
+            float wl[ZC_U], wb[ZC_U];
+#pragma unroll
+            for (int u = 0; u < ZC_U; ++u) {
+                wl[u] = vl[u]; wb[u] = vb[u];
+                x[u] = __ldg(reinterpret_cast<const float4 *>(Zk + (int64_t)cc[u] * 4));
+            }
+            if (j + ZC_U < width) entries(j + ZC_U);
+#pragma unroll
+            for (int u = 0; u < ZC_U; ++u) {
+                aL[0] = fmaf(wl[u], x[u].x, aL[0]); aL[1] = fmaf(wl[u], x[u].y, aL[1]);
+                aL[2] = fmaf(wl[u], x[u].z, aL[2]); aL[3] = fmaf(wl[u], x[u].w, aL[3]);
+                aB[0] = fmaf(wb[u], x[u].x, aB[0]); aB[1] = fmaf(wb[u], x[u].y, aB[1]);
+                aB[2] = fmaf(wb[u], x[u].z, aB[2]); aB[3] = fmaf(wb[u], x[u].w, aB[3]);
+            }
         }
         if (r >= n) continue;
         const int64_t o = r * 4;
@@ -325,12 +333,20 @@ __global__ void __launch_bounds__(256, 4) k_pcg_apply_zc(int64_t nwarps, int nch
             const float4 p4 = *reinterpret_cast<const float4 *>(Pk + o), q4 = *reinterpret_cast<const float4 *>(Qk + o);
             pr[0] = p4.x; pr[1] = p4.y; pr[2] = p4.z; pr[3] = p4.w;
             qr[0] = q4.x; qr[1] = q4.y; qr[2] = q4.z; qr[3] = q4.w;
+            if (D) {
+                const double *al = alpha_col + c0;
+                float4 *dp = reinterpret_cast<float4 *>(D + cbase + o), d4 = *dp;
+                d4.x = fmaf((float)__ldg(al), p4.x, d4.x); d4.y = fmaf((float)__ldg(al + 1), p4.y, d4.y);
+                d4.z = fmaf((float)__ldg(al + 2), p4.z, d4.z); d4.w = fmaf((float)__ldg(al + 3), p4.w, d4.w);
+                *dp = d4;
+            }
         }
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
-            const float tz = 0.5f * aL[w] - sh[w] * aB[w];
-            const float pn = first ? zr[w] : fmaf(bt[w], pr[w], zr[w]);
-            const float qn = first ? tz : fmaf(bt[w], qr[w], tz);
+            const float sh = (float)__ldg(shift + c0 + w), bt = first ? 0.f : (float)__ldg(beta_col + c0 + w);
+            const float tz = __fmaf_rn(0.5f, aL[w], -__fmul_rn(sh, aB[w]));
+            const float pn = first ? zr[w] : fmaf(bt, pr[w], zr[w]);
+            const float qn = first ? tz : fmaf(bt, qr[w], tz);
             pr[w] = pn; qr[w] = qn;
             contrib[w] = fmaf(pn, qn, contrib[w]);
         }
@@ -865,7 +881,7 @@ void launch_sell_spmm_colnorm(ofks_ctx *c, const T *val, const T *X, T *Y, doubl
 
 template <class T>
 void launch_pcg_apply(ofks_ctx *c, const T *valL, const T *valB, const T *Zin, int zc, T *P, T *Q, const double *beta_col,
-                      const double *shift, double *pq, int first, int w, int pc) {
+                      const double *shift, double *pq, int first, int w, int pc, T *Dlast, const double *alpha_col) {
     if constexpr (sizeof(T) == 4) {
         if (!zc && c->prm.pcg_staged && pcg_ws_fits(w)) {
             const unsigned grid = (unsigned)((c->n_slices + WS_WARPS - 1) / WS_WARPS);
@@ -886,9 +902,9 @@ void launch_pcg_apply(ofks_ctx *c, const T *valL, const T *valB, const T *Zin, i
             const int spw = spw_for((int64_t)c->n_tslices * nch);
             const int64_t nsg = ((int64_t)c->n_tslices + spw - 1) / spw, nw = nsg * nch;
             k_pcg_apply_zc<<<(unsigned)((nw * 32 + 255) / 256), 256, 0, c->stream>>>(
-                nw, nch, (int64_t)c->n_tslices, spw, pc, c->n, c->n_slots, c->d_tslice_ptr, c->d_tslice_w, c->d_tcols,
-                c->d_tvalL, c->d_tvalB, (const float *)Zin, (float *)P, (float *)Q, beta_col, shift,
-                c->d_cpart, first);
+                nw, nch, (int64_t)c->n_tslices, spw, c->n, c->n_slots, c->d_tslice_ptr, c->d_tslice_w, c->d_tcols,
+                c->d_tvalL, c->d_tvalB, (const float *)Zin, (float *)P, (float *)Q, (float *)Dlast,
+                alpha_col, beta_col, shift, c->d_cpart, first);
             c->kernels += 1;
             c->pq_units = nsg;
             return;
@@ -933,6 +949,7 @@ template void launch_sell_spmm<float>(ofks_ctx *, const float *, const float *, 
 template void launch_sell_spmm_colnorm<double>(ofks_ctx *, const double *, const double *, double *, double *);
 template void launch_sell_spmm_colnorm<float>(ofks_ctx *, const float *, const float *, float *, double *);
 template void launch_pcg_apply<double>(ofks_ctx *, const double *, const double *, const double *, int, double *,
-                                       double *, const double *, const double *, double *, int, int, int);
+                                       double *, const double *, const double *, double *, int, int, int, double *,
+                                       const double *);
 template void launch_pcg_apply<float>(ofks_ctx *, const float *, const float *, const float *, int, float *, float *,
-                                      const double *, const double *, double *, int, int, int);
+                                      const double *, const double *, double *, int, int, int, float *, const double *);
