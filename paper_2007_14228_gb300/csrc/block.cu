@@ -790,7 +790,6 @@ __global__ void __launch_bounds__(256) k_bb(int64_t n, int ld, int64_t stride, c
                                             const T *__restrict__ Xp, const T *__restrict__ D,
                                             const T *__restrict__ Dp, int have_prev, double *sc, double *gpart,
                                             unsigned *gcount) {
-    __shared__ double red[8];
     T sy = 0, yy = 0, ss = 0, xx = 0, dd = 0;
     {
         ELEM_BEGIN
@@ -802,9 +801,8 @@ __global__ void __launch_bounds__(256) k_bb(int64_t n, int ld, int64_t stride, c
             }
         ELEM_END
     }
-    const double tot[5] = {block_sum((double)sy, red), block_sum((double)yy, red), block_sum((double)ss, red),
-                           block_sum((double)xx, red), block_sum((double)dd, red)};
-    grid_accumulate<5>(tot, gpart, gcount, [&](int k, double v) {
+    const double tot[5] = {(double)sy, (double)yy, (double)ss, (double)xx, (double)dd};
+    grid_sums<5>(tot, gpart, gcount, [&](int k, double v) {
         sc[k < 3 ? SC_BB + k : (k == 3 ? SC_XNRM2 : SC_DNRM2)] = v;
     });
 }

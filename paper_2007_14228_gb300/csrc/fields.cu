@@ -200,7 +200,6 @@ __global__ void __launch_bounds__(256) k_rhs_gather(int64_t N, const int *__rest
 __global__ void __launch_bounds__(256) k_moments(int64_t N, const double *__restrict__ ynode,
                                                  const double *__restrict__ rhs, double *mom, double *gpart,
                                                  unsigned *gcount) {
-    __shared__ double sh[8];
     double m[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         const double r = rhs[i] * (1.0 / (4.0 * PI));
@@ -217,10 +216,7 @@ __global__ void __launch_bounds__(256) k_moments(int64_t N, const double *__rest
         m[8] = fma(r, 3.0 * y0 * y2, m[8]);
         m[9] = fma(r, 3.0 * y1 * y2, m[9]);
     }
-    double tot[10];
-#pragma unroll 1
-    for (int k = 0; k < 10; ++k) tot[k] = block_sum(m[k], sh);
-    grid_accumulate<10>(tot, gpart, gcount, [&](int k, double v) { mom[k] = v; });
+    grid_sums<10>(m, gpart, gcount, [&](int k, double v) { mom[k] = v; });
 }
 
 // Multipole boundary values V_B(r) = Q/|r| + d.r/|r|^3 + (1/2) sum Q_ij r_i r_j/|r|^5
