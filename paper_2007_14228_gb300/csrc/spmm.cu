@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(256) k_pcg_apply(int64_t nwarps, int nchunks, 
 #undef R_
 }
 
-constexpr int ZC_U = 7;                           // entries per pass of k_pcg_apply_zc
+constexpr int ZC_U = 4;                           // entries per pass of k_pcg_apply_zc
 
 // The float32 PCG apply on the type-grouped SELL with every PCG block chunk-major: element
 // (r, c) at ((c / 4) ns + r) 4 + c % 4 (ns = n rounded up to 32), rows in type order.  A warp
@@ -263,12 +263,12 @@ constexpr int ZC_U = 7;                           // entries per pass of k_pcg_a
 // bandwidth over, which the update pass does not (update 2.76 -> 2.42 ms in 32 iterations at n = 442k,
 // p = 41, 9.4 -> 7.4 in 16 at n = 493k, p = 210).
 //
-// What bounds it: L1 and L2 under the gathers.  ZC_U of them are in flight per lane at three CTAs per
-// SM, with the next pass's column ids and values behind them: 0.191 ms per launch at n = 442k with D
-// against 0.198 without D for four gathers, the rest of a row one by one, and four CTAs.  Four gathers
-// in this form at four CTAs 0.193, at three 0.236; two chunks per warp (an id and value pair for two
-// gathers, 80 or 118 registers) 0.188 to 0.214.
-__global__ void __launch_bounds__(256, 3) k_pcg_apply_zc(int64_t nwarps, int nchunks, int64_t n_slices, int spw,
+// What bounds it: L1 and L2 under the gathers.  ZC_U of them are in flight per lane at four CTAs per
+// SM, with the next pass's column ids and values behind them: with D 0.193 ms per launch at n = 442k and
+// 0.042 at n = 131k (without D, the rest of a row one by one, 0.198 and 0.044).  Seven gathers at three
+// CTAs 0.191 and 0.045, four at three CTAs 0.236 and 0.053; two chunks per warp (an id and value pair
+// for two gathers, 80 or 118 registers) 0.188 to 0.214 and 0.044 to 0.050.
+__global__ void __launch_bounds__(256, 4) k_pcg_apply_zc(int64_t nwarps, int nchunks, int64_t n_slices, int spw,
                                                       int64_t n, int64_t ns, const int *__restrict__ slice_ptr,
                                                       const int *__restrict__ slice_w,
                                                       const int *__restrict__ cols,
