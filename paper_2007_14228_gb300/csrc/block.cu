@@ -1005,7 +1005,7 @@ void launch_grad_update(ofks_ctx *c, Blocks<T> &b) {
             const int smw = (int)(sizeof(float) * (size_t)ld * (2 * GW_COLS + GW_PAD));
             const unsigned gw = (unsigned)(nsl * std::max<int64_t>(1, std::min<int64_t>((c->n + GW_ROWS - 1) / GW_ROWS,
                                                                                       152 / nsl)));
-            cudaFuncSetAttribute(k_grad_f32w, cudaFuncAttributeMaxDynamicSharedMemorySize, smw);
+            ofks_allow_smem((const void *)k_grad_f32w);
             k_grad_f32w<<<gw, 256, smw, c->stream>>>(c->n, c->p, ld, nsl, (const float *)b.HX, (const float *)b.BX,
                                                      c->d_C, c->d_L0, (float *)G, c->d_sc + SC_KKT2, c->d_gpart,
                                                      c->d_gcount);
@@ -1014,7 +1014,7 @@ void launch_grad_update(ofks_ctx *c, Blocks<T> &b) {
         if (ld <= 64) {
             const int smf = (int)(sizeof(float) * (2 * ld * ld + 64 * ld));
             const unsigned gf = (unsigned)std::max<int64_t>(1, std::min<int64_t>((c->n + 63) / 64, 152 * 4));
-#define GF_(k) { cudaFuncSetAttribute(k_grad_f32<k>, cudaFuncAttributeMaxDynamicSharedMemorySize, smf); \
+#define GF_(k) { ofks_allow_smem((const void *)k_grad_f32<k>); \
         k_grad_f32<k><<<gf, 256, smf, c->stream>>>(c->n, c->p, ld, (const float *)b.HX, (const float *)b.BX, \
                                                    c->d_C, c->d_L0, (float *)G, c->d_sc + SC_KKT2, c->d_gpart, \
                                                    c->d_gcount); }
@@ -1027,7 +1027,7 @@ void launch_grad_update(ofks_ctx *c, Blocks<T> &b) {
         if (launch_grad_dig(c, b.HX, b.BX, G, c->d_sc + SC_KKT2)) return;
     const unsigned grid = row_grid(32, c->n);
     const int no = (32 * ld + 255) / 256;
-#define GR_(k) { cudaFuncSetAttribute(k_grad<T, k>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
+#define GR_(k) { ofks_allow_smem((const void *)k_grad<T, k>); \
         k_grad<T, k><<<grid, 256, sm, c->stream>>>(c->n, c->p, ld, b.HX, b.BX, c->d_C, c->d_L0, G, \
                                                   c->d_sc + SC_KKT2, KC, c->d_gpart, c->d_gcount); }
     if (no <= 1) GR_(1) else if (no <= 2) GR_(2) else if (no <= 4) GR_(4) else if (no <= 6) GR_(6)
@@ -1206,7 +1206,7 @@ void launch_block_times_small(ofks_ctx *c, const T *X, const double *M, T *Y) {
     const size_t sm = sizeof(T) * (32 * ld + KC * ld);
     const unsigned grid = row_grid(32, c->n);
     MC_DISPATCH(mc_of(ld), {
-        cudaFuncSetAttribute(k_block_small<T, M_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        ofks_allow_smem((const void *)k_block_small<T, M_>);
         k_block_small<T, M_><<<grid, 256, sm, c->stream>>>(c->n, ld, X, M, Y, KC);
     });
 }

@@ -460,7 +460,7 @@ int cg_loop_run(ofks_ctx *c, double tol2, int *iters, int *status, double *rel2)
     const int want = std::max({P.nx, (P.ncol + P.NT - 1) / P.NT, (int)std::min<int64_t>(1 << 20, (rows + NTH - 1) / NTH)});
     const int grid = std::min(S.sms, want);
     auto kern = c->hartree_ff ? k_cg_loop<1> : k_cg_loop<0>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = ofks_allow_smem((const void *)kern);
     if (e == cudaSuccess) e = cudaMemsetAsync(S.loop_buf, 0, sizeof(double) * 8, c->stream);
     void *args[] = {&P};
     if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)grid), dim3(NTH), args, smem, c->stream);

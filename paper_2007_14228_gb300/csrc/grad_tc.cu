@@ -260,7 +260,7 @@ bool launch_grad_tc(ofks_ctx *c, const float *HX, const float *BX, float *G, dou
     if (smem > 220 * 1024) return false;
     const int64_t ntile = (c->n + RTM - 1) / RTM;
     const unsigned grid = (unsigned)(ntile < 152 ? ntile : 152);
-    cudaFuncSetAttribute(k_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    ofks_allow_smem((const void *)k_grad_tc);
     k_grad_tc<<<grid, 256, smem, c->stream>>>(c->n, c->p, ld, KP, nh, tcols, HX, BX, c->d_C, c->d_L0, G, kkt2,
                                               c->d_flag + 2, c->d_gpart, c->d_gcount);
     c->kernels += 1;

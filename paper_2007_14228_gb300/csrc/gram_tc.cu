@@ -240,7 +240,7 @@ bool launch_gram_tc(ofks_ctx *c, const float *X, const float *A, const float *B,
     const int64_t nslab = (c->n + GKS - 1) / GKS;
     // partials of 2 ld^2 doubles per CTA must fit the scratch (CPART_MIN >= 2 * 64^2 * 608)
     const unsigned grid = (unsigned)std::min<int64_t>(nslab, 152 * 4);
-    cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    ofks_allow_smem((const void *)k_gram_tc);
     k_gram_tc<<<grid, 256, smem, c->stream>>>(c->n, c->p, ld, nh, tcols, X, A, B, part, c->d_flag + 2);
     c->kernels += 1;
     *units = grid;

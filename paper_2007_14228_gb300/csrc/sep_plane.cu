@@ -170,7 +170,7 @@ int place_plane(const SepState &S, Plane &P, bool fwd) {
 template <class K, class Args>
 void go(ofks_ctx *c, K kern, Args &P, int items, int smem) {
     P.err = c->d_flag + 1;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    ofks_allow_smem((const void *)kern);
     kern<<<(unsigned)items, NT_, smem, c->stream>>>(P);
     c->kernels += 1;
 }

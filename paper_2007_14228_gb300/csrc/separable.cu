@@ -476,7 +476,7 @@ void sep_tc_launch(ofks_ctx *c, SepPass P) {
         smem = smem_for(2);
         gx = grid_for(smem);
     }
-    cudaFuncSetAttribute(k_sep_tc<SCALE, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    ofks_allow_smem((const void *)k_sep_tc<SCALE, SPLIT>);
     k_sep_tc<SCALE, SPLIT><<<dim3((unsigned)gx, (unsigned)d), 128, smem, c->stream>>>(P);
     c->kernels += 1;
 }
