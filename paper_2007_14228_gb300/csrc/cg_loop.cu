@@ -38,6 +38,11 @@ constexpr int NTH = 512, NW = NTH / 32;
 constexpr int BATCH = 8;                          // stencil entries whose loads are issued together
 constexpr int SPLIT_ROW = 40;                     // rows of more entries are shared by two lanes
 constexpr long long BAR_WAIT = 1LL << 21;
+// At least half of an SM's shared memory, so that two solves on streams of their own never share an
+// SM.  There, one solve's CTA could wait for tensor memory that the other's holds on one SM and hold
+// what the other's waits for on another, both behind their grid barriers.  Other kernels that use
+// tensor memory do not wait for other CTAs, so theirs is given back.
+constexpr uint32_t ALONE = 114 * 1024;
 
 struct CgOut {
     double rr, bb, rate;
@@ -426,7 +431,7 @@ int place_loop(const SepState &S, Loop &P) {
     P.lx = S.lx; P.lyzp = S.lyzp; P.T = S.t0;
     P.tcols = cols_of(std::max({tiles128(P.px) * P.NT, tiles128(P.pz) * P.py, tiles128(P.py) * P.pz}));
     const uint32_t need = o + 2 * std::max(P.part_p, P.part_m);
-    return need <= (uint32_t)(SMEM_MAX - 20 * 1024) && P.tcols <= 512 ? (int)need : 0;
+    return need <= (uint32_t)(SMEM_MAX - 20 * 1024) && P.tcols <= 512 ? (int)std::max(need, ALONE) : 0;
 }
 
 }  // namespace
