@@ -3,8 +3,9 @@
 // As kernels of their own (ten launches with the six-pass preconditioner) an iteration's phases cost
 // 112 us at 49^3 nodes, most of it launch latency, reloading the axis matrices and draining; here
 // one CTA per SM keeps the six axis matrices, the stencil tables and its tensor memory for the whole
-// solve, the phases are separated by grid barriers, and the residual test (with the iteration
-// counts it is taken at) runs on the device, so a solve is one launch and one host synchronization.
+// solve, the phases are separated by grid barriers, and the residual test runs on the device after
+// every iteration, so a solve is one launch and one host synchronization, and what it gives depends on
+// U, the right-hand side and the tolerance alone.
 //
 // The iteration is Chronopoulos and Gear's arrangement of CG (J. Comput. Appl. Math. 25, 1989): the
 // operator is applied to z = A_sep^-1 r instead of p, w = L z, and s = L p follows by recurrence,
@@ -45,7 +46,7 @@ constexpr long long BAR_WAIT = 1LL << 21;
 constexpr uint32_t ALONE = 114 * 1024;
 
 struct CgOut {
-    double rr, bb, rate;
+    double rr, bb;
     int it, status, abort;
     unsigned bar;
 };
@@ -67,7 +68,7 @@ struct Loop {
     const StencilCode *code;
     const double *val;
     const float2 *valff;
-    double tol2, rate;
+    double tol2;
     int max_iter;
     double *part;                                 // 4 x gridDim.x: zw, rr, rz, |rhs|^2
     CgOut *out;
@@ -92,12 +93,22 @@ __device__ __forceinline__ bool grid_barrier(CgOut *out, unsigned &target, int *
     return *s_abort == 0;
 }
 
-// sum of the CTAs' partials in CTA order, by every CTA
+// sum of the CTAs' partials in CTA order, by one warp of every CTA; the loads of the first 192 together
+__device__ __forceinline__ double warp_total(const double *part) {
+    constexpr int U = 6;
+    const unsigned lane = threadIdx.x & 31;
+    double v[U], s = 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = lane + 32 * u < gridDim.x ? __ldcg(part + lane + 32 * u) : 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) s += v[u];
+    for (unsigned i = lane + 32 * U; i < gridDim.x; i += 32) s += __ldcg(part + i);
+    return warp_sum(s);
+}
+
 __device__ __forceinline__ double grid_total(const double *part, double *s_val) {
     if (threadIdx.x < 32) {
-        double s = 0.0;
-        for (unsigned i = threadIdx.x; i < gridDim.x; i += 32) s += __ldcg(part + i);
-        s = warp_sum(s);
+        const double s = warp_total(part);
         if (threadIdx.x == 0) *s_val = s;
     }
     __syncthreads();
@@ -107,10 +118,7 @@ __device__ __forceinline__ double grid_total(const double *part, double *s_val) 
 // two such sums, one by each of the first two warps
 __device__ __forceinline__ void grid_totals(const double *p0, const double *p1, double *s_two) {
     if (threadIdx.x < 64) {
-        const double *part = threadIdx.x < 32 ? p0 : p1;
-        double s = 0.0;
-        for (unsigned i = threadIdx.x & 31; i < gridDim.x; i += 32) s += __ldcg(part + i);
-        s = warp_sum(s);
+        const double s = warp_total(threadIdx.x < 32 ? p0 : p1);
         if ((threadIdx.x & 31) == 0) s_two[threadIdx.x >> 5] = s;
     }
     __syncthreads();
@@ -206,8 +214,8 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
     __shared__ Tables tb;
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
-    __shared__ int abort_flag, s_abort, s_chunk;
-    __shared__ double sh[NW], s_val, s_coef, s_two[2], s_ab[2];
+    __shared__ int abort_flag, s_abort;
+    __shared__ double sh[NW], s_val, s_two[2], s_ab[2];
     __shared__ float s_l[64];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned G = gridDim.x;
@@ -258,8 +266,8 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
     ok = grid_barrier(P.out, target, &s_abort);
     const double bb = grid_total(part_bb, &s_val);
     __syncthreads();
-    double rr = grid_total(part_rr, &s_val), rr_prev = 0.0, rz = 0.0, rate = P.rate;
-    int it = 0, it_prev = 0, status = OFKS_OK;
+    double rr = grid_total(part_rr, &s_val), rz = 0.0;
+    int it = 0, status = OFKS_OK;
 
     // p = z + beta p, U += alpha p on the interior (warps over the rows along c) by CTAs c0, c0 + 1, ...
     auto direction = [&](double alpha, double beta, int c0) {
@@ -335,79 +343,55 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
     double alpha = 0.0, beta = 0.0;
     bool pending = false;
     while (ok) {
-        // the residual test, and the iterations to the next one: the count that the last observed
-        // factor of the squared residual predicts to the target, 1 to 8 (4 before any is known)
+        // the residual test, before every iteration: its sum is complete behind the last barrier
         if (!isfinite(rr)) { status = OFKS_ENONFINITE; break; }
-        if (rr <= P.tol2 * bb || bb == 0.0) {
-            if (it > it_prev && rr_prev > 0.0 && rr > 0.0 && rr < rr_prev) rate = pow(rr / rr_prev, 1.0 / (it - it_prev));
-            break;
-        }
+        if (rr <= P.tol2 * bb || bb == 0.0) break;
         if (it >= P.max_iter) { status = OFKS_ETIMEOUT; break; }
+        if (it == 0 && !(ok = forward(false, 0.0, 0.0))) break;
+        if (!(ok = backward(pending, alpha, beta))) break;
+        double zw = 0.0;
+        for_rows(P, tb,
+                 [&](const Row &R) {
+                     if constexpr (FF) {
+                         float s_hi = 0.f, s_lo = 0.f;
+                         row_product(tb, R, P.valff, 0.f, [&](int i) { return P.zf[i]; },
+                                     [&](float2 v, float x) { ff_madd(s_hi, s_lo, v, x); });
+                         return (double)s_hi + (double)s_lo;
+                     } else {
+                         double s = 0.0;
+                         row_product(tb, R, P.val, 0.0, [&](int i) { return P.V.z[i]; },
+                                     [&](double v, double x) { s = fma(v, x, s); });
+                         return s;
+                     }
+                 },
+                 [&](const Row &R, bool in, double s) {
+                     if (!in) return;
+                     P.q[R.node] = s;
+                     zw = fma(FF ? f2d_bits(P.zf[R.node]) : P.V.z[R.node], s, zw);
+                 });
+        const double tzw = cta_sum<NW>(zw, sh);
+        if (threadIdx.x == 0) part_zw[blockIdx.x] = tzw;
+        if (!(ok = grid_barrier(P.out, target, &s_abort))) break;
+        grid_totals(part_rz, part_zw, s_two);
         if (threadIdx.x == 0) {
-            double f = rate;
-            if (it > 0 && rr_prev > 0.0 && rr < rr_prev) f = pow(rr / rr_prev, 1.0 / (it - it_prev));
-            int chunk = 4;
-            if (f > 0.0 && f < 1.0) {
-                const double need = log(P.tol2 * bb / rr) / log(f);
-                chunk = (int)fmin(8.0, fmax(1.0, ceil(need)));
-            } else {
-                f = rate;
-            }
-            s_chunk = chunk;
-            s_coef = f;
+            const double b = it > 0 && rz > 0.0 ? s_two[0] / rz : 0.0;
+            const double den = alpha != 0.0 ? s_two[1] - b * s_two[0] / alpha : s_two[1];
+            s_ab[0] = den > 0.0 ? s_two[0] / den : 0.0;
+            s_ab[1] = b;
         }
         __syncthreads();
-        const int chunk = s_chunk;
-        rate = s_coef;
-        rr_prev = rr;
-        it_prev = it;
-        if (it == 0) ok = forward(false, 0.0, 0.0);
-        for (int j = 0; j < chunk && ok; ++j) {
-            if (!(ok = backward(pending, alpha, beta))) break;
-            double zw = 0.0;
-            for_rows(P, tb,
-                     [&](const Row &R) {
-                         if constexpr (FF) {
-                             float s_hi = 0.f, s_lo = 0.f;
-                             row_product(tb, R, P.valff, 0.f, [&](int i) { return P.zf[i]; },
-                                         [&](float2 v, float x) { ff_madd(s_hi, s_lo, v, x); });
-                             return (double)s_hi + (double)s_lo;
-                         } else {
-                             double s = 0.0;
-                             row_product(tb, R, P.val, 0.0, [&](int i) { return P.V.z[i]; },
-                                         [&](double v, double x) { s = fma(v, x, s); });
-                             return s;
-                         }
-                     },
-                     [&](const Row &R, bool in, double s) {
-                         if (!in) return;
-                         P.q[R.node] = s;
-                         zw = fma(FF ? f2d_bits(P.zf[R.node]) : P.V.z[R.node], s, zw);
-                     });
-            const double tzw = cta_sum<NW>(zw, sh);
-            if (threadIdx.x == 0) part_zw[blockIdx.x] = tzw;
-            if (!(ok = grid_barrier(P.out, target, &s_abort))) break;
-            grid_totals(part_rz, part_zw, s_two);
-            if (threadIdx.x == 0) {
-                const double b = it > 0 && rz > 0.0 ? s_two[0] / rz : 0.0;
-                const double den = alpha != 0.0 ? s_two[1] - b * s_two[0] / alpha : s_two[1];
-                s_ab[0] = den > 0.0 ? s_two[0] / den : 0.0;
-                s_ab[1] = b;
-            }
-            __syncthreads();
-            rz = s_two[0];
-            alpha = s_ab[0];
-            beta = s_ab[1];
-            ok = forward(true, alpha, beta);
-            pending = !spare;
-            ++it;
-        }
+        rz = s_two[0];
+        alpha = s_ab[0];
+        beta = s_ab[1];
+        ok = forward(true, alpha, beta);
+        pending = !spare;
+        ++it;
         if (ok) rr = grid_total(part_rr, &s_val);
         __syncthreads();
     }
     if (ok && pending) direction(alpha, beta, 0);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        P.out->rr = rr; P.out->bb = bb; P.out->rate = rate; P.out->it = it; P.out->status = status;
+        P.out->rr = rr; P.out->bb = bb; P.out->it = it; P.out->status = status;
     }
     cta_close(c, P.tcols, &P.out->abort);
 }
@@ -457,7 +441,7 @@ int cg_loop_run(ofks_ctx *c, double tol2, int *iters, int *status, double *rel2)
     P.p = c->d_cp; P.zf = reinterpret_cast<float *>(c->d_cz); P.q = c->d_cq; P.rhs = c->d_rhs;
     P.Lx = c->st.Lx;
     P.types = c->st.d_type; P.code = c->st.d_code; P.val = c->st.val; P.valff = c->st.valff;
-    P.tol2 = tol2; P.rate = c->cg_rate; P.max_iter = c->prm.poisson_max_iter;
+    P.tol2 = tol2; P.max_iter = c->prm.poisson_max_iter;
     P.out = reinterpret_cast<CgOut *>(S.loop_buf);
     P.part = S.loop_buf + 8;
     // CTAs: one per SM, fewer where the mesh has too few planes, tiles and rows to feed them
@@ -475,7 +459,6 @@ int cg_loop_run(ofks_ctx *c, double tol2, int *iters, int *status, double *rel2)
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return ofks_cuda_check(c, e, "Hartree CG");
     if (h.abort) return ofks_fail(c, OFKS_ETIMEOUT, "Hartree CG: a bounded device wait timed out");
-    c->cg_rate = h.rate;
     *iters = h.it;
     *status = h.status;
     *rel2 = h.bb > 0.0 ? h.rr / h.bb : 0.0;

@@ -244,7 +244,7 @@ struct ofks_ctx {
     int k = 0;
     int cg_last = 0;                             // CG iterations of the last Hartree solve
     double cg_rate = 0.0;                        // per-iteration factor of the squared Hartree CG residual
-                                                 // observed in the last solve (0: none yet)
+                                                 // observed in the last solve by separate kernels (0: none yet)
     double hartree_tol = 0.0;                    // > 0: tolerance of the next Hartree solve (adaptive mode)
     bool hartree_ff = false;                     // this Hartree solve keeps p as float32 pairs (d_cpff) too
     int64_t cg_total = 0;                        // ... summed since the counter was cleared
