@@ -432,8 +432,9 @@ bool cg_loop_fits(const SepState &S) {
 
 // Solves L U = rhs on the interior from U's current values and boundary data to
 // |r|^2 <= tol2 |rhs|^2; iterations and status (OFKS_OK, OFKS_ETIMEOUT at max_iter,
-// OFKS_ENONFINITE, or an error) on return.  One launch, one synchronization.
-int cg_loop_run(ofks_ctx *c, double tol2, int *iters, int *status, double *rel2) {
+// OFKS_ENONFINITE, or an error) on return.  One launch, one synchronization.  *ran is false, and nothing is
+// done, where the device does not take the grid at once (fewer SMs at hand than it reports).
+int cg_loop_run(ofks_ctx *c, double tol2, bool *ran, int *iters, int *status, double *rel2) {
     SepState &S = c->sep;
     Loop P{};
     const int smem = place_loop(S, P);
@@ -453,6 +454,11 @@ int cg_loop_run(ofks_ctx *c, double tol2, int *iters, int *status, double *rel2)
     if (e == cudaSuccess) e = cudaMemsetAsync(S.loop_buf, 0, sizeof(double) * 8, c->stream);
     void *args[] = {&P};
     if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)grid), dim3(NTH), args, smem, c->stream);
+    *ran = e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported;
+    if (!*ran) {
+        cudaGetLastError();
+        return OFKS_OK;
+    }
     c->kernels += 1;
     CgOut h;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h, P.out, sizeof(h), cudaMemcpyDeviceToHost, c->stream);

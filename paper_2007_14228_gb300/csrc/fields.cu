@@ -571,12 +571,13 @@ int run_hartree(ofks_ctx *c) {
     // during the float32 iterations the lattice SpMV of the separable CG runs in float-float
     // arithmetic (~48 bits, its tolerance is at least poisson_tol_mixed); float64 otherwise
     c->hartree_ff = sep && lat && c->phase == 32 && c->st.valff != nullptr;
-    if (sep && lat && c->sep.loop && c->prm.poisson_sep_tc) {
-        int iters = 0, status = OFKS_OK;
-        double rel2 = 0.0;
+    bool ran = false;                                   // the persistent form; else its passes as kernels
+    int iters = 0, status = OFKS_OK;
+    double rel2 = 0.0;
+    if (sep && lat && c->sep.loop && c->prm.poisson_sep_tc)
+        if (const int rc = cg_loop_run(c, tol2, &ran, &iters, &status, &rel2)) return rc;
+    if (ran) {
         c->kernels += 1;
-        const int rc = cg_loop_run(c, tol2, &iters, &status, &rel2);
-        if (rc) return rc;
         if (status == OFKS_ENONFINITE) return ofks_fail(c, status, "Hartree CG residual is not finite");
         if (status == OFKS_ETIMEOUT)
             return ofks_fail(c, status, "Hartree CG: %d iterations, relative residual %.3e", iters, std::sqrt(rel2));

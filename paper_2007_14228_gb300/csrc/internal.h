@@ -336,7 +336,7 @@ bool sep_plane_fits(const SepState &S);
 constexpr int64_t CG_LOOP_MAX_N = 600000;
 bool cg_loop_fits(const SepState &S);
 int64_t cg_loop_doubles(int sms);
-int cg_loop_run(ofks_ctx *c, double tol2, int *iters, int *status, double *rel2);
+int cg_loop_run(ofks_ctx *c, double tol2, bool *ran, int *iters, int *status, double *rel2);
 void sep_plane_hartree(ofks_ctx *c, int it, int slot, int first);
 
 // ---- fields.cu (density, potentials, Hamiltonian refresh, Poisson)

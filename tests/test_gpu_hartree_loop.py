@@ -1,5 +1,8 @@
 """The persistent Hartree CG: what a solve depends on, where it stops, and what follows a failure."""
+import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -7,6 +10,8 @@ import pytest
 from paper_2007_14228_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -64,3 +69,48 @@ def test_the_iteration_limit_is_kept(ofks, limit):
     assert e.value.code == ofks.ETIMEOUT
     assert int(re.search(r"Hartree CG: (\d+) iterations", str(e.value)).group(1)) == limit
     ctx.close()
+
+
+REFUSE = """
+int cudaLaunchCooperativeKernel(const void *f, ...) { return 720; }   /* cudaErrorCooperativeLaunchTooLarge */
+"""
+
+CHILD = """
+import sys
+import numpy as np
+from paper_2007_14228_gb300 import inputs as I, ofks
+s = I.lih().with_cells((9, 8, 10))
+m = I.make_mesh(s)
+out = {}
+for precision in ("fp64", "mixed"):
+    ctx = ofks.context_for(s, m, beta=10.0, precision=precision, poisson_tol_mixed=1e-12)
+    ctx.init_orbitals(I.initial_block(m.n_free, s.p, 0))
+    r = ctx.evaluate()
+    out[precision] = ctx.get_field("U")
+    out["its_" + precision] = r["hartree_iters"]
+    ctx.step(2)
+    out["X_" + precision] = ctx.get_orbitals()
+    ctx.close()
+np.savez(sys.argv[1], **out)
+"""
+
+
+# two solves to a 1e-12 relative residual agree within 1e-9 of the potential's norm, the iterates within 1e-8
+# (the bounds of the parity tests); float32 iterates within the float32 forms' 5e-5
+def test_a_refused_launch_falls_back_to_separate_kernels(ofks, tmp_path):
+    src, so = tmp_path / "refuse.c", tmp_path / "refuse.so"
+    src.write_text(REFUSE)
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
+    runs = []
+    for env in ({}, {"LD_PRELOAD": str(so)}):
+        path = str(tmp_path / f"out{len(runs)}.npz")
+        r = subprocess.run([sys.executable, "-c", CHILD, path], cwd=ROOT, env=dict(os.environ, **env),
+                           capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-2000:]
+        runs.append(np.load(path))
+    a, b = runs
+    for precision, bound in (("fp64", 1e-8), ("mixed", 5e-5)):
+        assert 0 < b["its_" + precision] < 60
+        assert np.linalg.norm(a[precision] - b[precision]) <= 1e-9 * np.linalg.norm(a[precision])
+        X, Y = a["X_" + precision], b["X_" + precision]
+        assert np.linalg.norm(X - Y) <= bound * np.linalg.norm(X)
