@@ -349,6 +349,7 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
         if (it >= P.max_iter) { status = OFKS_ETIMEOUT; break; }
         if (it == 0 && !(ok = forward(false, 0.0, 0.0))) break;
         if (!(ok = backward(pending, alpha, beta))) break;
+        pending = false;
         double zw = 0.0;
         for_rows(P, tb,
                  [&](const Row &R) {
@@ -374,15 +375,19 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
         if (!(ok = grid_barrier(P.out, target, &s_abort))) break;
         grid_totals(part_rz, part_zw, s_two);
         if (threadIdx.x == 0) {
-            const double b = it > 0 && rz > 0.0 ? s_two[0] / rz : 0.0;
-            const double den = alpha != 0.0 ? s_two[1] - b * s_two[0] / alpha : s_two[1];
-            s_ab[0] = den > 0.0 ? s_two[0] / den : 0.0;
+            double b = it > 0 ? s_two[0] / rz : 0.0;
+            double den = it > 0 ? s_two[1] - b * s_two[0] / alpha : s_two[1];
+            if (!(den > 0.0)) { b = 0.0; den = s_two[1]; }   // the recurrence is lost: again from p = z
+            s_ab[0] = s_two[0] > 0.0 && den > 0.0 ? s_two[0] / den : 0.0;
             s_ab[1] = b;
         }
         __syncthreads();
         rz = s_two[0];
         alpha = s_ab[0];
         beta = s_ab[1];
+        // no descent along z either (r.z or z.w not positive: z has no value beside its rounding, or r is
+        // beyond float32): nothing that follows would differ
+        if (alpha == 0.0) { status = isfinite(s_two[0]) && isfinite(s_two[1]) ? OFKS_ETIMEOUT : OFKS_ENONFINITE; break; }
         ok = forward(true, alpha, beta);
         pending = !spare;
         ++it;

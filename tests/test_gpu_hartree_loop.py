@@ -114,3 +114,21 @@ def test_a_refused_launch_falls_back_to_separate_kernels(ofks, tmp_path):
         assert np.linalg.norm(a[precision] - b[precision]) <= 1e-9 * np.linalg.norm(a[precision])
         X, Y = a["X_" + precision], b["X_" + precision]
         assert np.linalg.norm(X - Y) <= bound * np.linalg.norm(X)
+
+
+# A density beyond float32's range: the preconditioner's operands overflow or vanish, and no step along them
+# exists.  The solve says so at once, and the context goes on with a block that it can solve for.
+@pytest.mark.parametrize("scale,code", [(1e30, "ENONFINITE"), (1e-40, "ETIMEOUT")])
+def test_a_solve_without_a_direction_ends(ofks, scale, code):
+    s, m, V = lih((8, 8, 8))
+    ctx = ofks.context_for(s, m, beta=10.0, xc=0)
+    ctx.set_orbitals(V * scale)
+    with pytest.raises(ofks.OfksError) as e:
+        ctx.evaluate()
+    assert e.value.code == getattr(ofks, code), e.value
+    its = re.search(r"Hartree CG: (\d+) iterations", str(e.value))
+    assert its is None or int(its.group(1)) < 100
+    ctx.set_orbitals(V)
+    r = ctx.evaluate()
+    assert 0 < r["hartree_iters"] < 60
+    ctx.close()
