@@ -132,3 +132,32 @@ def test_a_solve_without_a_direction_ends(ofks, scale, code):
     r = ctx.evaluate()
     assert 0 < r["hartree_iters"] < 60
     ctx.close()
+
+
+# The first solve after a failed one starts from what that left in U, and ends where a new context's does.
+@pytest.mark.parametrize("cells", [(8, 8, 8), (24, 24, 24), (80, 40, 41)], ids=str)
+def test_recovery_after_each_failure(ofks, cells):
+    s, m, V = lih(cells)
+    x = m.xyz[m.free_ids()]
+    V = np.stack([np.exp(-2.0 * np.linalg.norm(x, axis=1)), x[:, 0] * np.exp(-0.7 * np.linalg.norm(x, axis=1))], axis=1)
+    ctx = ofks.context_for(s, m, beta=10.0)
+    ctx.init_orbitals(V)
+    X = ctx.get_orbitals()
+    ctx.evaluate()
+    ref = ctx.get_field("U")
+    ctx.close()
+    bad = X.copy()
+    bad[len(bad) // 2, 0] = np.inf
+    ctx = ofks.context_for(s, m, beta=10.0)
+    for block, limit, code in ((X, 1, ofks.ETIMEOUT), (bad, 100, ofks.ENONFINITE), (X * 1.3, 2, ofks.ETIMEOUT)):
+        ctx.set_params(poisson_max_iter=limit)
+        ctx.set_orbitals(block)
+        with pytest.raises(ofks.OfksError) as e:
+            ctx.evaluate()
+        assert e.value.code == code
+        ctx.set_params(poisson_max_iter=100)
+        ctx.set_orbitals(X)
+        assert ctx.evaluate()["hartree_iters"] < 60   # none where the failure left the potential as it was
+        U = ctx.get_field("U")
+        assert np.linalg.norm(U - ref) <= 1e-9 * np.linalg.norm(ref)
+    ctx.close()
