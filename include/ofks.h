@@ -409,7 +409,9 @@ int ofks_load_state(ofks_ctx *ctx, const char *path);
 
 /* Per-kernel device time accumulated while profiling is on (CUDA events around each
  * launch of the named kernel family).  on = 1 starts (and clears), 0 stops.  While it is on
- * the CUDA graphs are not used (every launch runs on its own between its events). */
+ * the CUDA graphs are not used (every launch runs on its own between its events).  Where the Hartree
+ * solve is one launch, poisson_spmv and poisson_pc hold that launch's phases, one per CG iteration, by the
+ * device's clock (the vector updates ride in the latter, and poisson_vec stays empty). */
 int ofks_profile(ofks_ctx *ctx, int32_t on);
 /* kernel family id -> launches and total milliseconds since profiling was switched on;
  * name (may be NULL) receives a static string. */

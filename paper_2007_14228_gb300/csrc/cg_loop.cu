@@ -49,7 +49,9 @@ struct CgOut {
     double rr, bb;
     int it, status, abort;
     unsigned bar;
+    unsigned long long ns[2];                     // profiling: nanoseconds of the SpMV, of the passes
 };
+static_assert(sizeof(CgOut) <= 8 * sizeof(double), "room in cg_loop_doubles");
 
 struct Loop {
     int nx, ny, nz, px, py, pz, ncol, NT;
@@ -70,6 +72,7 @@ struct Loop {
     const float2 *valff;
     double tol2;
     int max_iter;
+    int timed;                                    // profiling is on
     double *part;                                 // 4 x gridDim.x: zw, rr, rz, |rhs|^2
     CgOut *out;
 };
@@ -340,8 +343,20 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
         return grid_barrier(P.out, target, &s_abort);
     };
 
+    // profiling: the time since the last call goes to phase k, by one thread of the grid
+    unsigned long long t_last = 0, t_ns[2] = {0, 0};
+    const bool clock = P.timed && blockIdx.x == 0 && threadIdx.x == 0;
+    auto lap = [&](int k) {
+        if (!clock) return;
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        if (k >= 0) t_ns[k] += t - t_last;
+        t_last = t;
+    };
+
     double alpha = 0.0, beta = 0.0;
     bool pending = false;
+    lap(-1);
     while (ok) {
         // the residual test, before every iteration: its sum is complete behind the last barrier
         if (!isfinite(rr)) { status = OFKS_ENONFINITE; break; }
@@ -350,6 +365,7 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
         if (it == 0 && !(ok = forward(false, 0.0, 0.0))) break;
         if (!(ok = backward(pending, alpha, beta))) break;
         pending = false;
+        lap(1);
         double zw = 0.0;
         for_rows(P, tb,
                  [&](const Row &R) {
@@ -373,6 +389,7 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
         const double tzw = cta_sum<NW>(zw, sh);
         if (threadIdx.x == 0) part_zw[blockIdx.x] = tzw;
         if (!(ok = grid_barrier(P.out, target, &s_abort))) break;
+        lap(0);
         grid_totals(part_rz, part_zw, s_two);
         if (threadIdx.x == 0) {
             double b = it > 0 ? s_two[0] / rz : 0.0;
@@ -393,10 +410,12 @@ __global__ void __launch_bounds__(NTH, 1) k_cg_loop(const Loop P) {
         ++it;
         if (ok) rr = grid_total(part_rr, &s_val);
         __syncthreads();
+        lap(1);
     }
     if (ok && pending) direction(alpha, beta, 0);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         P.out->rr = rr; P.out->bb = bb; P.out->it = it; P.out->status = status;
+        P.out->ns[0] = t_ns[0]; P.out->ns[1] = t_ns[1];
     }
     cta_close(c, P.tcols, &P.out->abort);
 }
@@ -447,7 +466,7 @@ int cg_loop_run(ofks_ctx *c, double tol2, bool *ran, int *iters, int *status, do
     P.p = c->d_cp; P.zf = reinterpret_cast<float *>(c->d_cz); P.q = c->d_cq; P.rhs = c->d_rhs;
     P.Lx = c->st.Lx;
     P.types = c->st.d_type; P.code = c->st.d_code; P.val = c->st.val; P.valff = c->st.valff;
-    P.tol2 = tol2; P.max_iter = c->prm.poisson_max_iter;
+    P.tol2 = tol2; P.max_iter = c->prm.poisson_max_iter; P.timed = c->prof ? 1 : 0;
     P.out = reinterpret_cast<CgOut *>(S.loop_buf);
     P.part = S.loop_buf + 8;
     // CTAs: one per SM, fewer where the mesh has too few planes, tiles and rows to feed them
@@ -470,6 +489,10 @@ int cg_loop_run(ofks_ctx *c, double tol2, bool *ran, int *iters, int *status, do
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return ofks_cuda_check(c, e, "Hartree CG");
     if (h.abort) return ofks_fail(c, OFKS_ETIMEOUT, "Hartree CG: a bounded device wait timed out");
+    if (c->prof) {                                // the phases of the one launch, by the device's clock
+        c->prof_n[PF_POISSON_SPMV] += h.it; c->prof_ms[PF_POISSON_SPMV] += 1e-6 * (double)h.ns[0];
+        c->prof_n[PF_POISSON_PC] += h.it; c->prof_ms[PF_POISSON_PC] += 1e-6 * (double)h.ns[1];
+    }
     *iters = h.it;
     *status = h.status;
     *rel2 = h.bb > 0.0 ? h.rr / h.bb : 0.0;

@@ -161,3 +161,21 @@ def test_recovery_after_each_failure(ofks, cells):
         U = ctx.get_field("U")
         assert np.linalg.norm(U - ref) <= 1e-9 * np.linalg.norm(ref)
     ctx.close()
+
+
+# bounds: the phases lie inside the launch, whose start (the first residual) is in neither; the device's clock
+# ticks every 32 ns or, at the coarsest, every microsecond
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_the_profile_holds_the_phases_of_the_solve(ofks, precision):
+    s, m, V = lih((24, 24, 24))
+    ctx = ofks.context_for(s, m, beta=10.0, precision=precision)
+    ctx.init_orbitals(V)
+    ctx.profile(True)
+    its = ctx.evaluate()["hartree_iters"]
+    prof = ctx.profile_get()
+    ctx.profile(False)
+    ctx.close()
+    spmv, passes, whole = (prof[k] for k in ("poisson_spmv", "poisson_pc", "poisson"))
+    assert spmv["launches"] == passes["launches"] == its > 0
+    assert spmv["ms"] > 0 and passes["ms"] > 0
+    assert 0.5 * whole["ms"] < spmv["ms"] + passes["ms"] < whole["ms"] + 1e-3 * 3 * its
