@@ -65,7 +65,7 @@ __device__ __forceinline__ double combine(long long hi, long long lo, int e) {
     const int ex = 63 - lz + SH + e + 1023;
     unsigned long long bits = ((unsigned long long)ex << 52) + (mant - 0x10000000000000ull);
     if (ex <= 0) bits = 0;
-    if (ex >= 2046) bits = 0x7ff0000000000000ull;
+    if (ex >= 2047) bits = 0x7ff0000000000000ull;
     return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
