@@ -1,16 +1,26 @@
-// float64 products on the bf16 tensor cores by exact digits.
+// float64 products on the bf16 tensor cores by integer digits.
 //
 // A vector of float64 values with largest biased exponent e is held as 61-bit integers
 // f = round(v 2^(1083 - e)), |f| < 2^61 (values within eight binades of the largest are exact), and
 // these as seven balanced digits of nine bits, f = sum_s q_s 2^(9 (6 - s)), |q_s| <= 256, which bf16
 // holds exactly.  Digit products are integers below 2^16, so a float32 accumulator adds them exactly
 // while their sum stays below 2^24; products with s + t = d share an accumulator, and d = 0 .. 6 are
-// kept (what is dropped is below 2^-58 of the product of the two largest magnitudes, per term,
-// against float64's own rounding of 2^-53).  The seven accumulators v_d of an entry are combined in
-// integers, T = sum_d v_d 2^(9 (6 - d)), and rounded once to float64: no float64 arithmetic, which on
-// GB300 takes 16 cycles per warp instruction.
+// kept.  The seven accumulators v_d of an entry are combined in integers, T = sum_d v_d 2^(9 (6 - d)),
+// and rounded once to float64: no float64 arithmetic, which on GB300 takes 16 cycles per warp
+// instruction.
 //
-// A vector that holds an infinity or a NaN is marked by exponent 2047; its results are NaN.
+// Error: a term loses six digit products of up to 2^16 at weight 2^45 and less below, and up to half a
+// unit of either f times the other, together below 7.01 2^61 where the product of the two largest
+// magnitudes is 2^120 at least.  The accumulator d = 6 passes 2^24 from 43 terms on, and a unit lost there
+// weighs 2^54.  A sum of p <= 48 terms is therefore off by at most
+//   7.2 p 2^-59 x (power of two of the first vector's largest) x (that of the second's).
+// For entries far smaller than that, which a float64 sum would hold to 2^-53 of their own
+// terms, the callers compare it with sum |a||b| and add in float64 where it is too coarse: `magnitude`
+// gives the bf16 factors of one more product that bounds the sum of magnitudes from below.
+//
+// A vector that holds an infinity or a NaN has exponent 2047, one of subnormal values only counts as 1,
+// and 0 means that all are zero; the callers do not use the digits where values or results could be
+// subnormal or infinite.
 #pragma once
 
 #include <stdint.h>
@@ -22,6 +32,12 @@ namespace dig {
 constexpr int ND = 7;                             // digits
 
 __device__ __forceinline__ int exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+__device__ __forceinline__ bool nonzero(double v) { return (__double_as_longlong(v) << 1) != 0; }
+
+// |v| 2^(1023 - e) cut to eight bits, as bf16 bits: zero below 2^-126 (e >= 128), at most 2^60
+__device__ __forceinline__ uint32_t magnitude(double v, int e) {
+    return (uint32_t)min(max(((__double2hiint(v) & 0x7fffffff) >> 13) - ((e - 127) << 7), 0), 187 << 7);
+}
 
 // the seven digits of v against the largest exponent e of its vector, as the high halves of float32
 // bit patterns (bf16), digit s in q[s]
@@ -41,7 +57,8 @@ __device__ __forceinline__ void split(double v, int e, uint32_t (&q)[ND]) {
     }
 }
 
-// (hi 2^SH + lo) 2^e rounded to float64 (to nearest, ties away from zero; subnormal results are zero)
+// (hi 2^SH + lo) 2^e rounded to float64 (to nearest, ties away from zero; subnormal results, which the
+// callers do not ask for, are zero)
 template <int SH>
 __device__ __forceinline__ double combine(long long hi, long long lo, int e) {
     constexpr uint32_t LOW = SH == 32 ? 0xffffffffu : (1u << (SH & 31)) - 1u;

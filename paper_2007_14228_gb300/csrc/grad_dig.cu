@@ -1,18 +1,28 @@
 // The float64 gradient G = H X + B X C and the residual norm |H X - B X Lambda0|_F (Alg. 2, Sec. 4.1)
-// on the tensor cores: B X and [C | Lambda0] as exact digits (digits.cuh), 28 digit products per
-// contraction.
+// on the tensor cores: B X and [C | Lambda0] without their diagonals as integer digits (digits.cuh), 28
+// digit products per contraction; the diagonals' terms are one float64 multiply-add each.
 //
 // What bounds it: the direct form issues 2 ld float64 multiply-adds per entry on a pipe that takes 16
-// cycles for a warp's, 84 % of that pipe's peak; here an entry takes three float64 operations, and the
-// rest is integer work on the digits (75 instructions per entry of B X, ~60 per output) and the
-// readback of seven accumulators: 7.51 -> 1.43 ms at n = 1.18 M, p = 41; 2.83 -> 0.56 at n = 442k;
-// 0.164 -> 0.077 at n = 68k, p = 23.
+// cycles for a warp's, 84 % of that pipe's peak; here an entry takes five float64 operations, and the
+// rest is integer work on the digits (80 instructions per entry of B X, ~65 per output) and the
+// readback of eight accumulators: 7.51 -> 1.89 ms at n = 1.18 M, p = 41; 2.83 -> 0.73 at n = 442k;
+// 0.164 -> 0.099 at n = 68k, p = 23.
+//
+// Accuracy, entry by entry: the digits are off by at most 7.2 p 2^-59 of the product of the row's largest
+// magnitude and the column's largest off the diagonal, the direct form's p multiply-adds by p 2^-53 of
+// sum_k |B X_rk| |C_kc|.  A twenty-ninth product, of the magnitudes cut to eight bits with the diagonal,
+// bounds that sum from below; where it is less than 7.2/64 of the two largest (a row whose large entries
+// meet small ones of C), and for rows or columns beyond the digits' range, the products are added up in
+// float64.  So no entry's bound is larger than the direct form's.  The diagonal stays out because it is
+// often far larger than the rest of its column (blocks close to eigenvectors, or noise: 3.6 ms at n = 442k,
+// p = 41 with most entries added up, 0.73 so); on smooth blocks and noise none to 1e-5 of the entries are added
+// up, on columns that share few rows nearly all may be, which then costs as much as the direct form does.
 //
 // One persistent CTA per SM walks 128-row tiles.  Two threads per row load it, agree on its largest
-// exponent and write its seven digits as K-major operands; one thread issues the products of B X
-// with C, 7 accumulators of nh columns in tensor memory; every warp reads its 32 rows and half of
-// the columns back, combines, adds H X and stores G; then the same with Lambda0 for the norm.  The next
-// tile's rows are loaded meanwhile.  Every wait is bounded, as in grad_tc.cu.
+// exponent and write its seven digits and magnitudes as K-major operands; one thread issues the products
+// of B X with C, 8 accumulators of nh columns in tensor memory; every warp reads its 32 rows and half of
+// the columns back, combines, adds H X and the diagonal's term and stores G; then the same with Lambda0
+// for the norm.  The next tile's rows are loaded meanwhile.  Every wait is bounded, as in grad_tc.cu.
 #include <algorithm>
 
 #include "digits.cuh"
@@ -22,6 +32,10 @@ namespace {
 using namespace sepp;
 
 constexpr int OT = 128, OTH = 256;                // rows per tile, threads
+constexpr int NS = dig::ND + 1;                   // operands of a block: its digits and its magnitudes
+constexpr float FINE = 7.2f / 64.f;               // least sum of magnitudes for which the digits stand
+// exponents that the digits stand for: no infinities, and no subnormal values, products or results
+__device__ __forceinline__ bool usable(int e) { return e == 0 || (e >= 575 && e < 2047); }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t addr, float *v) {
     uint32_t u[8];
@@ -44,8 +58,12 @@ __global__ void __launch_bounds__(OTH, 1) k_grad_dig(int64_t n, int p, int ld, i
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag, sE[OT], sEC[2][nh];
+    __shared__ float sLeast[2][nh];                   // per column, the least sum of magnitudes
+    __shared__ double sDiag[2][nh];                   // the diagonals
     __shared__ double red[OTH / 32];
-    const uint32_t sA = su32(dsm), sB = sA + dig::ND * AB;          // digits of B X; of C and Lambda0
+    constexpr int PX = nh + 2;                                     // pitch of sX: rows 16 bytes apart in the banks
+    const uint32_t sA = su32(dsm), sB = sA + NS * AB;              // operands of B X; of C and Lambda0
+    double *sX = reinterpret_cast<double *>(dsm + NS * AB + 2 * NS * BB);   // the tile of B X
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t ntile = (n + OT - 1) / OT;
     Cta c;
@@ -56,19 +74,25 @@ __global__ void __launch_bounds__(OTH, 1) k_grad_dig(int64_t n, int p, int ld, i
         const int col = e < nh ? e : e - nh;
         int mx = 0;
         if (col < p)
-            for (int k = 0; k < p; ++k) mx = max(mx, dig::exponent(M[(int64_t)k * ld + col]));
+            for (int k = 0; k < p; ++k) {
+                const double v = k == col ? 0.0 : M[(int64_t)k * ld + col];
+                mx = max(mx, max(dig::exponent(v), dig::nonzero(v) ? 1 : 0));
+            }
         sEC[e < nh ? 0 : 1][col] = mx;
+        sDiag[e < nh ? 0 : 1][col] = col < p ? M[(int64_t)col * ld + col] : 0.0;
+        sLeast[e < nh ? 0 : 1][col] = mx == 0 ? -1.f : usable(mx) ? FINE : INFINITY;
     }
     __syncthreads();
     for (int e = tid; e < 2 * nh * nh; e += OTH) {
         const int m = e / (nh * nh), k = (e - m * nh * nh) / nh, col = e % nh;
         const double *M = m == 0 ? C : L0;
+        const double v = k < p && col < p ? M[(int64_t)k * ld + col] : 0.0;
         uint32_t q[dig::ND];
-        dig::split(k < p && col < p ? M[(int64_t)k * ld + col] : 0.0, sEC[m][col], q);
+        dig::split(k != col ? v : 0.0, sEC[m][col], q);
 #pragma unroll
-        for (int s = 0; s < dig::ND; ++s)
-            *reinterpret_cast<uint16_t *>(dsm + dig::ND * AB + (uint32_t)(m * dig::ND + s) * BB + coff<LBA>(col, k, k8)) =
-                (uint16_t)q[s];
+        for (int s = 0; s < NS; ++s)
+            *reinterpret_cast<uint16_t *>(dsm + NS * AB + (uint32_t)(m * NS + s) * BB + coff<LBA>(col, k, k8)) =
+                (uint16_t)(s < dig::ND ? q[s] : dig::magnitude(v, sEC[m][col]));
     }
     const int crow = tid >> 1, ccol = (tid & 1) * HALF;             // this thread's part of a row to convert
     double x[HALF];
@@ -81,20 +105,21 @@ __global__ void __launch_bounds__(OTH, 1) k_grad_dig(int64_t n, int p, int ld, i
             x[j] = v.x; x[j + 1] = v.y;
         }
     };
-    // products of the tile's digits with matrix m, the seven accumulators side by side
-    auto multiply = [&](int m) -> bool {
+    // products of the tile's digits with matrix m, the seven accumulators side by side, and of the magnitudes
+    auto multiply = [&](int m) {
         asm volatile("fence.proxy.async.shared::cta;");
         asm volatile("tcgen05.fence::before_thread_sync;");
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;");
         if (tid == 0) {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nh >> 3) << 17) | (8u << 24);
-            for (int d = 0; d < dig::ND; ++d)
-                for (int s = 0; s <= d; ++s)
+            for (int d = 0; d < NS; ++d)
+                for (int s = d < dig::ND ? 0 : d; s <= d; ++s)
                     for (int kk = 0; kk < NH; ++kk) {
+                        const int t = d < dig::ND ? d - s : d;
                         const uint64_t ad = sdesc(sA + s * AB + kk * 2 * LBA, LBA, k8 * LBA);
-                        const uint64_t bd = sdesc(sB + (uint32_t)(m * dig::ND + d - s) * BB + kk * 2 * LBA, LBA, k8 * LBA);
-                        const uint32_t accum = (s > 0 || kk > 0) ? 1u : 0u;
+                        const uint64_t bd = sdesc(sB + (uint32_t)(m * NS + t) * BB + kk * 2 * LBA, LBA, k8 * LBA);
+                        const uint32_t accum = ((d < dig::ND && s > 0) || kk > 0) ? 1u : 0u;
                         asm volatile(
                             "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(c.tmem + d * nh),
@@ -102,7 +127,6 @@ __global__ void __launch_bounds__(OTH, 1) k_grad_dig(int64_t n, int p, int ld, i
                     }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(c.mbar));
         }
-        return true;
     };
     auto wait = [&]() -> bool {
         uint32_t done = 0;
@@ -119,16 +143,45 @@ __global__ void __launch_bounds__(OTH, 1) k_grad_dig(int64_t n, int p, int ld, i
     };
     double part = 0.0;
     const int row = (warp & 3) * 32 + lane, col0 = (warp >> 2) * HALF;   // this thread's outputs of a tile
+    // the coarse columns of row r in float64, four at a time (rare; a warp's four columns cost what they do in
+    // the direct form)
+    auto direct = [&](int m, int64_t r, unsigned coarse) {
+        const double *M = m == 0 ? C : L0;
+#pragma unroll 1
+        for (int q = 0; q < HALF && col0 + q < ld; q += 4) {
+            if (!__any_sync(0xffffffffu, coarse >> q & 15u)) continue;
+            double t[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int k = 0; k < p; ++k) {
+                const double b = r < n ? BX[r * ld + k] : 0.0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) t[j] = fma(b, __ldg(M + (int64_t)k * ld + col0 + q + j), t[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int col = col0 + q + j;
+                if (!(coarse >> (q + j) & 1u) || col >= p) continue;
+                const double hx = HX[r * ld + col];
+                if (m == 0) G[r * ld + col] = hx + t[j];
+                else part = fma(hx - t[j], hx - t[j], part);
+            }
+        }
+    };
     if (blockIdx.x < ntile) fetch(blockIdx.x);
     for (int64_t tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
         int mx = 0;
 #pragma unroll
         for (int j = 0; j < HALF; ++j) mx = max(mx, dig::exponent(x[j]));
+        if (mx == 0)
+#pragma unroll
+            for (int j = 0; j < HALF; ++j) mx |= dig::nonzero(x[j]) ? 1 : 0;
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
         if ((tid & 1) == 0) sE[crow] = mx;
 #pragma unroll
+        for (int j = 0; j < HALF; j += 2)
+            *reinterpret_cast<double2 *>(sX + crow * PX + ccol + j) = make_double2(x[j], x[j + 1]);
+#pragma unroll
         for (int g = 0; g < NH; ++g) {
-            uint32_t w[dig::ND][4];
+            uint32_t w[NS][4];
 #pragma unroll
             for (int j = 0; j < 8; j += 2) {
                 uint32_t a[dig::ND], b[dig::ND];
@@ -136,9 +189,10 @@ __global__ void __launch_bounds__(OTH, 1) k_grad_dig(int64_t n, int p, int ld, i
                 dig::split(x[8 * g + j + 1], mx, b);
 #pragma unroll
                 for (int s = 0; s < dig::ND; ++s) w[s][j >> 1] = a[s] | (b[s] << 16);
+                w[dig::ND][j >> 1] = dig::magnitude(x[8 * g + j], mx) | (dig::magnitude(x[8 * g + j + 1], mx) << 16);
             }
 #pragma unroll
-            for (int s = 0; s < dig::ND; ++s)
+            for (int s = 0; s < NS; ++s)
                 st16(sA + s * AB + coff<LBA>(crow, ccol + 8 * g, k8), make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]));
         }
         multiply(0);
@@ -151,17 +205,25 @@ __global__ void __launch_bounds__(OTH, 1) k_grad_dig(int64_t n, int p, int ld, i
             h[j] = v.x; h[j + 1] = v.y;
         }
         const int eR = sE[row];                       // written before multiply's barrier
+        const float lift = eR == 0 ? FINE : 0.f;      // a zero row's products are zero
         for (int m = 0; m < 2; ++m) {
             if (!wait()) break;
             if (m == 1 && tile + gridDim.x < ntile) fetch(tile + gridDim.x);
+            unsigned coarse = usable(eR) ? 0u : ~0u;  // the thread's columns whose digits are too coarse
 #pragma unroll
             for (int cb = 0; cb < HALF; cb += 8) {
-                float v[dig::ND][8];
+                float v[NS][8];
 #pragma unroll
-                for (int d = 0; d < dig::ND; ++d)
+                for (int d = 0; d < NS; ++d)
                     tmem_ld8(c.tmem + ((uint32_t)((warp & 3) * 32) << 16) + d * nh + col0 + cb, v[d]);
                 asm volatile("tcgen05.wait::ld.sync.aligned;");
-                double g[8];
+                double g[8], b[8];
+                if (m == 0)
+#pragma unroll
+                    for (int j = 0; j < 8; j += 2) {
+                        const double2 t = *reinterpret_cast<const double2 *>(sX + row * PX + col0 + cb + j);
+                        b[j] = t.x; b[j + 1] = t.y;
+                    }
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     long long hi = 0, lo = 0;
@@ -169,12 +231,13 @@ __global__ void __launch_bounds__(OTH, 1) k_grad_dig(int64_t n, int p, int ld, i
                     for (int d = 0; d < 4; ++d) hi = (hi << 9) + (int)v[d][j];
 #pragma unroll
                     for (int d = 4; d < dig::ND; ++d) lo = (lo << 9) + (int)v[d][j];
-                    const int eC = sEC[m][col0 + cb + j];
-                    double val = dig::combine<27>(hi, lo, eR + eC - 2 * 1083 + 54);
-                    if (eR == 2047 || eC == 2047) val = __longlong_as_double(0x7ff8000000000000ll);
                     const int col = col0 + cb + j;
-                    if (m == 0) g[j] = h[cb + j] + val;
-                    else if (col < p && r < n) {
+                    const double val = dig::combine<27>(hi, lo, eR + sEC[m][col] - 2 * 1083 + 54);
+                    if (v[dig::ND][j] + lift < sLeast[m][col]) coarse |= 1u << (cb + j);
+                    if (m == 0) {
+                        g[j] = h[cb + j] + fma(b[j], sDiag[0][col], val);
+                        h[cb + j] = fma(-b[j], sDiag[1][col], h[cb + j]);
+                    } else if (col < p && r < n && !(coarse >> (cb + j) & 1u)) {
                         const double res = h[cb + j] - val;
                         part = fma(res, res, part);
                     }
@@ -185,6 +248,8 @@ __global__ void __launch_bounds__(OTH, 1) k_grad_dig(int64_t n, int p, int ld, i
                         if (col0 + cb + j < ld)
                             *reinterpret_cast<double2 *>(G + r * ld + col0 + cb + j) = make_double2(g[j], g[j + 1]);
             }
+            if (r >= n) coarse = 0u;
+            if (__any_sync(0xffffffffu, coarse != 0u)) direct(m, r, coarse);
             if (m == 0) multiply(1);                  // its barrier follows the last read of the accumulators
         }
         if (abort_flag) break;
@@ -203,8 +268,8 @@ bool launch_grad_dig(ofks_ctx *c, const double *HX, const double *BX, double *G,
     const int ld = c->ld;
     if (ld % 4 || ld < GRAD_DIG_MIN || ld > 48) return false;
     const int NH = (ld + 15) / 16, nh = 16 * NH;
-    const int tcols = cols_of(dig::ND * nh);
-    const uint32_t k8 = nh / 8, smem = dig::ND * (OT / 8 * k8 * LBA) + 2 * dig::ND * (nh / 8 * k8 * LBA);
+    const int tcols = cols_of(NS * nh);
+    const uint32_t k8 = nh / 8, smem = NS * (OT / 8 * k8 * LBA) + 2 * NS * (nh / 8 * k8 * LBA) + 8 * OT * (nh + 2);
     const int64_t ntile = (c->n + OT - 1) / OT;
     const unsigned grid = (unsigned)std::min<int64_t>(ntile, 152);
     // tensor memory for one CTA per SM where it takes more than half of the columns

@@ -371,8 +371,8 @@ bool launch_gram_tc(ofks_ctx *c, const float *X, const float *A, const float *B,
 // grad_tc.cu: G = H X + B X C and |H X - B X Lambda0|^2 on the tensor cores (false: not supported)
 bool launch_grad_tc(ofks_ctx *c, const float *HX, const float *BX, float *G, double *kkt2);
 // float64 gradient by digit products on the tensor cores (grad_dig.cu), GRAD_DIG_MIN <= ld <= 48: below,
-// the direct form's 2 ld multiply-adds per entry cost no more than the digits; above, the digits of a
-// tile, of C and of Lambda0 do not fit in shared memory
+// the direct form's 2 ld multiply-adds per entry cost no more than the digits; above, the operands of a
+// tile, of C and of Lambda0 do not fit in shared memory (64 columns: 322 KB)
 constexpr int GRAD_DIG_MIN = 16;
 bool launch_grad_dig(ofks_ctx *c, const double *HX, const double *BX, double *G, double *kkt2);
 // float64 Grams by digit products (gram_dig.cu), ld >= GRAM_DIG_MIN (below, the direct form's ld multiply-adds
