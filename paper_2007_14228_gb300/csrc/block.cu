@@ -20,14 +20,16 @@ namespace {
 // Rows are staged KR at a time in shared memory.
 // The block's partial tile (its split of the rows) goes to part, entry-major: the value of
 // tile entry (m, a, b) of tile pair q at part[((q 2 + m) TS + a) TS + b) splits + split], and
-// k_gram_fin adds the splits in order.
+// k_gram_fin adds the splits in order.  With `when`, nothing is done unless it is set (the digit form's
+// entries hold).
 template <class T, int RT>
 __global__ void __launch_bounds__(256) k_gram2(int64_t n, int p, int ld, int ntile,
                                                const T *__restrict__ X,
                                                const T *__restrict__ A,
                                                const T *__restrict__ B, double *part,
-                                               int64_t rows_per_split) {
+                                               int64_t rows_per_split, const int *when) {
     constexpr int TS = 16 * RT, KR = 16;
+    if (when && *when == 0) return;
     __shared__ T xs[KR][TS], as[KR][TS], bs[KR][TS];
     // decode the upper-triangular tile pair
     const int q = blockIdx.x;
@@ -182,9 +184,12 @@ __global__ void __launch_bounds__(256) k_gram_f32w(int64_t n, int p, int ld, int
 
 // The Grams from the split partials: one warp per upper entry (m, i <= j < p) adds its units
 // (splits) in order (lanes stride, then a fixed butterfly) and writes the entry and its mirror.
-// Tiles of TS x TS, ntile per side, pairs numbered row by row over the upper triangle.
+// Tiles of TS x TS, ntile per side, pairs numbered row by row over the upper triangle.  With slack
+// (gram_dig.cu) a total below GRAM_DIG_LEAST sets *redo; without it but with redo, nothing is done unless that is set.
 __global__ void __launch_bounds__(256) k_gram_fin(int p, int ld, int TS, int ntile, int64_t units,
-                                                  const double *__restrict__ part, double *XA, double *XB) {
+                                                  const double *__restrict__ part, double *XA, double *XB,
+                                                  const float *__restrict__ slack, int *redo) {
+    if (!slack && redo && *redo == 0) return;
     const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int64_t nup = (int64_t)p * (p + 1) / 2;
@@ -201,6 +206,11 @@ __global__ void __launch_bounds__(256) k_gram_fin(int p, int ld, int TS, int nti
     double s = 0.0;
     for (int64_t u = lane; u < units; u += 32) s += __ldcg(a + u);
     s = warp_sum(s);
+    if (slack) {
+        float t = 0.f;
+        for (int64_t u = lane; u < units; u += 32) t += __ldcg(slack + e * units + u);
+        if (!(warp_sum_f(t) >= GRAM_DIG_LEAST) && lane == 0) *redo = 1;
+    }
     if (lane == 0) {
         double *M = m == 0 ? XA : XB;
         M[(int64_t)i * ld + j] = s;
@@ -932,10 +942,16 @@ void launch_gram2(ofks_ctx *c, const T *X, const T *A, const T *B, double *XA, d
     cudaMemsetAsync(XA, 0, sizeof(double) * ld * ld, c->stream);    // the padding stays zero
     cudaMemsetAsync(XB, 0, sizeof(double) * ld * ld, c->stream);
     // the split partials are added in split order by k_gram_fin (one warp per upper entry)
-    auto fin = [&](int TS, int ntile, int64_t units) {
+    auto fin = [&](int TS, int ntile, int64_t units, const float *slack = nullptr, int *redo = nullptr) {
         const int64_t warps = (int64_t)p * (p + 1);
         k_gram_fin<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, c->stream>>>(p, ld, TS, ntile, units, c->d_cpart,
-                                                                               XA, XB);
+                                                                               XA, XB, slack, redo);
+    };
+    auto direct = [&](int TS, int ntile, int64_t splits, int64_t rps, const int *when) {
+        const dim3 grid((unsigned)(ntile * (ntile + 1) / 2), (unsigned)splits);
+#define G_(rt) k_gram2<T, rt><<<grid, 256, 0, c->stream>>>(c->n, p, ld, ntile, X, A, B, c->d_cpart, rps, when)
+        switch (TS / 16) { case 1: G_(1); break; case 2: G_(2); break; case 3: G_(3); break; default: G_(4); }
+#undef G_
     };
     if constexpr (sizeof(T) == 4) {
         int64_t units = 0;
@@ -955,10 +971,12 @@ void launch_gram2(ofks_ctx *c, const T *X, const T *A, const T *B, double *XA, d
         }
     }
     if constexpr (sizeof(T) == 8) {
-        int ts = 0, nt = 0;
-        int64_t units = 0;
-        if (launch_gram_dig(c, X, A, B, c->d_cpart, &ts, &nt, &units)) {
-            fin(ts, nt, units);
+        GramDig f;
+        if (launch_gram_dig(c, X, A, B, c->d_cpart, &f)) {
+            fin(f.ts, f.ntile, f.splits, f.slack, f.redo);
+            direct(f.ts, f.ntile, f.splits, f.rps, f.redo);         // both idle unless the flag is set
+            fin(f.ts, f.ntile, f.splits, nullptr, f.redo);
+            c->kernels += 2;
             return;
         }
     }
@@ -967,10 +985,7 @@ void launch_gram2(ofks_ctx *c, const T *X, const T *A, const T *B, double *XA, d
     int64_t splits = std::max<int64_t>(1, std::min<int64_t>((c->n + 255) / 256, (152LL * 4) / npair + 1));
     const int64_t rps = ((c->n + splits - 1) / splits + 15) / 16 * 16;
     splits = (c->n + rps - 1) / rps;
-    dim3 grid((unsigned)npair, (unsigned)splits);
-#define G_(rt) k_gram2<T, rt><<<grid, 256, 0, c->stream>>>(c->n, p, ld, ntile, X, A, B, c->d_cpart, rps)
-    switch (RT) { case 1: G_(1); break; case 2: G_(2); break; case 3: G_(3); break; default: G_(4); }
-#undef G_
+    direct(TS, ntile, splits, rps, nullptr);
     fin(TS, ntile, splits);
 }
 

@@ -224,7 +224,7 @@ struct ofks_ctx {
     int *d_gmap = nullptr;                       // learned preconditioner: active column ids [ld]
     double *d_sc = nullptr;                      // SC_COUNT scalars
     double *d_rec = nullptr;                     // iteration record (device)
-    int *d_flag = nullptr;                       // error / status flags
+    int *d_flag = nullptr;                       // status of the last p x p kernel, timeouts (2), GramDig::redo
     // deterministic reductions (common.cuh): grid_accumulate partials (GACC_CAP doubles) and its
     // block counter; per-column partials [column][unit] of the block kernels (cpart_cap doubles)
     double *d_gpart = nullptr;
@@ -378,8 +378,15 @@ bool launch_grad_dig(ofks_ctx *c, const double *HX, const double *BX, double *G,
 // float64 Grams by digit products (gram_dig.cu), ld >= GRAM_DIG_MIN (below, the direct form's ld multiply-adds
 // per entry cost no more than the digits): partials for k_gram_fin
 constexpr int GRAM_DIG_MIN = 16;
-bool launch_gram_dig(ofks_ctx *c, const double *X, const double *A, const double *B, double *part, int *ts, int *ntile,
-                     int64_t *units);
+// least total slack of an entry: what it leaves out, products of the largest below 2^-126, is nothing beside
+constexpr float GRAM_DIG_LEAST = 0x1p-100f;
+struct GramDig {
+    int ts = 0, ntile = 0;                       // tiles of ts columns, ntile per side
+    int64_t splits = 0, rps = 0;                 // ranges of rps rows
+    float *slack = nullptr;                      // per partial, how far its digits are from too coarse
+    int *redo = nullptr;                         // set by k_gram_fin where an entry's are (device)
+};
+bool launch_gram_dig(ofks_ctx *c, const double *X, const double *A, const double *B, double *part, GramDig *f);
 template <class T> void launch_grad_update(ofks_ctx *c, Blocks<T> &b);
 // The PCG's working set: its block width w (row pitch of R, Z, P, Q, W and of the D it builds,
 // and the stride of its per-column arrays cb) and its real column count pc.  In the compact

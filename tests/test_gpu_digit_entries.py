@@ -96,20 +96,50 @@ def test_every_entry_of_the_gradient(ofks, p, kind):
     assert np.all(np.abs(G - ref) <= 1.001 * bound + 1e-307 * 2.0 ** -40)
 
 
+# Lambda0 = X^T H X and S = X^T B X: sums of 64 rows by digits, or direct sums over at most 128 rows, added over
+# the ranges of rows
+@pytest.mark.parametrize("kind", ["plain", "spikes", "localized", "graded"])
+@pytest.mark.parametrize("p", [13, 16, 17, 23, 32, 33, 41, 48, 49, 64, 65, 97, 129])
+def test_every_entry_of_the_grams(ofks, p, kind):
+    s = I.lih().with_cells((8, 7, 6)).with_p(p, occ=1.0)
+    m = I.make_mesh(s)
+    X = block(m, p, kind)
+    f = fields(ofks, s, m, X, ("HX", "BX", "Lambda0", "S"), xc=0)
+    for A, got in ((f["HX"], f["Lambda0"]), (f["BX"], f["S"])):
+        ref = np.triu(X.astype(Q).T @ A.astype(Q))
+        ref = ref + np.triu(ref, 1).T
+        bound = (128 + len(X) / 64 + 3) * 2.0 ** -53 * np.triu(np.abs(X).T @ np.abs(A))
+        bound = np.maximum(bound, bound.T)
+        assert np.all(np.abs(got - ref) <= 1.001 * bound + 1e-307 * 2.0 ** -40)
+
+
 # an infinity gives the infinities and NaNs of the direct sum
-def test_infinities_of_the_gradient(ofks):
-    p = 17
+def test_infinities_of_the_grams(ofks):
+    p, j = 17, 3
     s = I.lih().with_cells((6, 4, 5)).with_p(p, occ=1.0)
     m = I.make_mesh(s)
     X = block(m, p, "plain")
-    X[5, 3] = np.inf
-    f = fields(ofks, s, m, X, ("HX", "BX", "G", "S", "Lambda"), xc=0, method="moptqr")
-    C = -f["Lambda"]
+    ctx = ofks.context_for(s, m, beta=10.0)
+    e = np.zeros_like(X)
+    # a node with the most neighbours: its row has no padding entries, whose zeros would give NaN
+    x = m.xyz[m.free_ids()]
+    best, count = 0, 0
+    for r in np.argsort(np.linalg.norm(x - x.mean(axis=0), axis=1))[:16]:
+        e[:, 0] = 0.0
+        e[r, 0] = 1.0
+        c = np.count_nonzero(ctx.apply("B", e)[:, 0])
+        if c > count:
+            best, count = r, c
+    e[:, 0] = 0.0
+    e[best, 0] = 1.0
+    col = ctx.apply("B", e)[:, 0]
+    ctx.close()
+    X[:, j] = np.where(col < 0, -1.0, 1.0)        # every product with the column's infinities has one sign
+    X[best, j] = np.inf
+    f = fields(ofks, s, m, X, ("BX", "S"), xc=0)
     with np.errstate(invalid="ignore", over="ignore"):
-        # no NaN where every product is an infinity of one sign or finite
-        parts = np.concatenate([f["HX"][:, None, :], f["BX"][:, :, None] * C[None, :, :]], axis=1)
-        ref = parts.sum(axis=1)
-    assert np.isinf(ref).any() or np.isnan(ref).any()
-    assert np.array_equal(np.isnan(f["G"]), np.isnan(ref))
+        ref = np.array([[np.sum(X[:, min(a, b)] * f["BX"][:, max(a, b)]) for b in range(p)] for a in range(p)])
+    assert np.isinf(ref).sum() > p // 2
+    assert np.array_equal(np.isnan(f["S"]), np.isnan(ref))
     inf = np.isinf(ref)
-    assert np.array_equal(f["G"][inf], ref[inf])
+    assert np.array_equal(f["S"][inf], ref[inf])
