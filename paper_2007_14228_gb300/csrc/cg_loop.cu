@@ -20,8 +20,9 @@
 // Measured against the usual arrangement (SpMV on p, five barriers), Hartree solves of four steps: 8^3
 // cells 2.46 -> 2.38 ms, 24^3 3.41 -> 3.15, 21x19x23 3.40 -> 3.20, 60x32x30 (float-float) 4.45 -> 4.01.
 // float64 operations of a warp take 16 cycles each, so the
-// passes that run on few SMs hold as few of them as possible.  512 threads and eight loads in
-// flight per lane measured best (44 and 92 us per iteration in the usual arrangement; 256: 50 us at 49^3 and 120 at 121x65x61; 768: 49 and 102).
+// passes that run on few SMs hold as few of them as possible.  An iteration of a cold solve at 8^3, 24^3 and
+// 60x32x30 cells takes 28.6, 39.5 and 77.9 us with 512 threads, 29.3, 44.8 and 106 with 256, 32.6, 44.4 and
+// 84.6 with 768 (separate kernels: 72, 88 and 131).
 //
 // Sums over the grid go through one partial per CTA, written before a barrier and added in CTA
 // order by every CTA after it.  A barrier wait is bounded: on timeout the CTA raises the abort

@@ -330,9 +330,11 @@ bool sep_pcg_ready(ofks_ctx *c, int w);                        // separable PCG 
 void sep_pcg_passes(ofks_ctx *c, int w, const double *shift);  // z = T_sep^-1 r on the PCG tensor
 // the Hartree step in three passes (sep_plane.cu)
 bool sep_plane_fits(const SepState &S);
-// The whole Hartree CG as one persistent kernel (cg_loop.cu), up to CG_LOOP_MAX_N interior nodes: on
-// the largest meshes that its shared memory admits beyond that, the SpMV at one CTA per SM loses
-// against its own kernel at full occupancy what the launches cost.
+// The whole Hartree CG as one persistent kernel (cg_loop.cu), up to CG_LOOP_MAX_N interior nodes: what it
+// saves shrinks with the mesh, since its SpMV runs at one CTA per SM.  An evaluation by separate kernels
+// against by this one, float64 and mixed, p = 2: 493k nodes 4.13 -> 3.55 and 2.70 -> 2.32 ms, 614k 4.77 -> 4.40 and
+// 3.23 -> 2.86, 753k 5.47 -> 5.36 and 3.61 -> 3.48, 857k 5.92 -> 6.03 and 3.96 -> 3.77; the line is drawn well
+// before the float64 form loses.
 constexpr int64_t CG_LOOP_MAX_N = 600000;
 bool cg_loop_fits(const SepState &S);
 int64_t cg_loop_doubles(int sms);
@@ -371,12 +373,14 @@ bool launch_gram_tc(ofks_ctx *c, const float *X, const float *A, const float *B,
 // grad_tc.cu: G = H X + B X C and |H X - B X Lambda0|^2 on the tensor cores (false: not supported)
 bool launch_grad_tc(ofks_ctx *c, const float *HX, const float *BX, float *G, double *kkt2);
 // float64 gradient by digit products on the tensor cores (grad_dig.cu), GRAD_DIG_MIN <= ld <= 48: below,
-// the direct form's 2 ld multiply-adds per entry cost no more than the digits; above, the operands of a
+// the direct form's 2 ld multiply-adds per entry cost no more than the digits (n = 442k, direct and digits: ld = 12
+// 0.250 and 0.265 ms, 16 0.409 and 0.275; n = 68k: 0.062 and 0.058, 0.088 and 0.060); above, the operands of a
 // tile, of C and of Lambda0 do not fit in shared memory (64 columns: 322 KB)
 constexpr int GRAD_DIG_MIN = 16;
 bool launch_grad_dig(ofks_ctx *c, const double *HX, const double *BX, double *G, double *kkt2);
 // float64 Grams by digit products (gram_dig.cu), ld >= GRAM_DIG_MIN (below, the direct form's ld multiply-adds
-// per entry cost no more than the digits): partials for k_gram_fin
+// per entry cost about what the digits do; n = 442k, direct and digits: ld = 8 0.129 and 0.158 ms, 12 0.175 and
+// 0.164, 16 0.256 and 0.164): partials for k_gram_fin
 constexpr int GRAM_DIG_MIN = 16;
 // least total slack of an entry: what it leaves out, products of the largest below 2^-126, is nothing beside
 constexpr float GRAM_DIG_LEAST = 0x1p-100f;

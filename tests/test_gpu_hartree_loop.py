@@ -179,3 +179,30 @@ def test_the_profile_holds_the_phases_of_the_solve(ofks, precision):
     assert spmv["launches"] == passes["launches"] == its > 0
     assert spmv["ms"] > 0 and passes["ms"] > 0
     assert 0.5 * whole["ms"] < spmv["ms"] + passes["ms"] < whole["ms"] + 1e-3 * 3 * its
+
+
+# The form that a mesh takes, told by the launches of a solve: the persistent form one, the separate kernels five
+# per CG iteration (SpMV, three passes, direction) or, with an axis too long for these, ten (six contractions,
+# the update with its gather, a scatter).  The extents are those at which the forms are compared elsewhere.
+@pytest.mark.parametrize("cells,form", [((6, 4, 4), "loop"), ((8, 8, 8), "loop"), ((24, 24, 24), "loop"), ((64, 6, 5), "loop"),
+                                        ((65, 9, 7), "loop"), ((6, 5, 65), "loop"), ((6, 64, 65), "three"),
+                                        ((100, 5, 6), "three"), ((6, 70, 72), "three"), ((80, 40, 41), "three"),
+                                        ((6, 96, 97), "six")], ids=str)
+def test_the_form_of_a_solve(ofks, cells, form):
+    s, m, V = lih(cells)
+    launches = {}
+    for hartree in (0, 1):
+        ctx = ofks.context_for(s, m, beta=10.0, hartree=hartree)
+        ctx.init_orbitals(V)
+        ctx.profile(True)
+        its = ctx.evaluate()["hartree_iters"]
+        launches[hartree] = ctx.profile_get()["all_kernels"]["launches"]
+        ctx.close()
+    extra = launches[1] - launches[0]
+    assert its > 3
+    if form == "loop":
+        assert extra <= 8
+    elif form == "three":
+        assert 5 * its <= extra <= 5 * its + 12
+    else:
+        assert 10 * its <= extra <= 10 * its + 20
