@@ -40,11 +40,8 @@ int ofks_cuda_check(ofks_ctx *c, cudaError_t e, const char *what) {
     return ofks_fail(c, OFKS_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
-cudaError_t ofks_allow_smem(const void *kern) {
-    cudaFuncAttributes a;
-    cudaError_t e = cudaFuncGetAttributes(&a, kern);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)a.sharedSizeBytes);
+cudaError_t ofks_allow_smem(const void *kern, int own) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - own);
 }
 
 static cudaEvent_t ev_get(ofks_ctx *c) {

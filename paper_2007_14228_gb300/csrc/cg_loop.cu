@@ -45,6 +45,7 @@ constexpr long long BAR_WAIT = 1LL << 21;
 // what the other's waits for on another, both behind their grid barriers.  Other kernels that use
 // tensor memory do not wait for other CTAs, so theirs is given back.
 constexpr uint32_t ALONE = 114 * 1024;
+constexpr int OWN = 20 * 1024;                    // at least the kernel's static shared memory
 
 struct CgOut {
     double rr, bb;
@@ -440,7 +441,7 @@ int place_loop(const SepState &S, Loop &P) {
     P.lx = S.lx; P.lyzp = S.lyzp; P.T = S.t0;
     P.tcols = cols_of(std::max({tiles128(P.px) * P.NT, tiles128(P.pz) * P.py, tiles128(P.py) * P.pz}));
     const uint32_t need = o + 2 * std::max(P.part_p, P.part_m);
-    return need <= (uint32_t)(SMEM_MAX - 20 * 1024) && P.tcols <= 512 ? (int)std::max(need, ALONE) : 0;
+    return need <= (uint32_t)(SMEM_MAX - OWN) && P.tcols <= 512 ? (int)std::max(need, ALONE) : 0;
 }
 
 }  // namespace
@@ -475,7 +476,7 @@ int cg_loop_run(ofks_ctx *c, double tol2, bool *ran, int *iters, int *status, do
     const int want = std::max({P.nx, (P.ncol + P.NT - 1) / P.NT, (int)std::min<int64_t>(1 << 20, (rows + NTH - 1) / NTH)});
     const int grid = std::min(S.sms, want);
     auto kern = c->hartree_ff ? k_cg_loop<1> : k_cg_loop<0>;
-    cudaError_t e = ofks_allow_smem((const void *)kern);
+    cudaError_t e = ofks_allow_smem((const void *)kern, OWN);
     if (e == cudaSuccess) e = cudaMemsetAsync(S.loop_buf, 0, sizeof(double) * 8, c->stream);
     void *args[] = {&P};
     if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)grid), dim3(NTH), args, smem, c->stream);

@@ -282,10 +282,10 @@ struct ofks_ctx {
 // ---- helpers (api.cu)
 int ofks_fail(ofks_ctx *c, int code, const char *fmt, ...);
 int ofks_cuda_check(ofks_ctx *c, cudaError_t e, const char *what);
-// Allows a kernel the most dynamic shared memory that its own static shared memory leaves.  The limit
-// belongs to the kernel, not to a context: set to what one launch needs, a thread with a smaller mesh
-// or block could lower it between another's call and launch.
-cudaError_t ofks_allow_smem(const void *kern);
+// Allows a kernel the most dynamic shared memory that its static shared memory, at most `own` bytes, leaves.
+// The limit belongs to the kernel, not to a context: set to what one launch needs, a thread with a smaller
+// mesh or block could lower it between another's call and launch.
+cudaError_t ofks_allow_smem(const void *kern, int own = 1024);
 void prof_begin(ofks_ctx *c, int fam, cudaEvent_t *a, cudaEvent_t *b);
 void prof_end(ofks_ctx *c, int fam, cudaEvent_t a, cudaEvent_t b);
 
