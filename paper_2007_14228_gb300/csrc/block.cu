@@ -947,11 +947,18 @@ void launch_gram2(ofks_ctx *c, const T *X, const T *A, const T *B, double *XA, d
         k_gram_fin<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, c->stream>>>(p, ld, TS, ntile, units, c->d_cpart,
                                                                                XA, XB, slack, redo);
     };
-    auto direct = [&](int TS, int ntile, int64_t splits, int64_t rps, const int *when) {
-        const dim3 grid((unsigned)(ntile * (ntile + 1) / 2), (unsigned)splits);
+    // the CUDA-core form, with `when` only where that is set
+    auto direct = [&](int *when) {
+        const int RT = p <= 16 ? 1 : (p <= 32 ? 2 : (p <= 48 ? 3 : 4));
+        const int TS = 16 * RT, ntile = (p + TS - 1) / TS, npair = ntile * (ntile + 1) / 2;
+        int64_t splits = std::max<int64_t>(1, std::min<int64_t>((c->n + 255) / 256, (152LL * 4) / npair + 1));
+        const int64_t rps = ((c->n + splits - 1) / splits + 15) / 16 * 16;
+        splits = (c->n + rps - 1) / rps;
+        const dim3 grid((unsigned)npair, (unsigned)splits);
 #define G_(rt) k_gram2<T, rt><<<grid, 256, 0, c->stream>>>(c->n, p, ld, ntile, X, A, B, c->d_cpart, rps, when)
-        switch (TS / 16) { case 1: G_(1); break; case 2: G_(2); break; case 3: G_(3); break; default: G_(4); }
+        switch (RT) { case 1: G_(1); break; case 2: G_(2); break; case 3: G_(3); break; default: G_(4); }
 #undef G_
+        fin(TS, ntile, splits, nullptr, when);
     };
     if constexpr (sizeof(T) == 4) {
         int64_t units = 0;
@@ -974,19 +981,12 @@ void launch_gram2(ofks_ctx *c, const T *X, const T *A, const T *B, double *XA, d
         GramDig f;
         if (launch_gram_dig(c, X, A, B, c->d_cpart, &f)) {
             fin(f.ts, f.ntile, f.splits, f.slack, f.redo);
-            direct(f.ts, f.ntile, f.splits, f.rps, f.redo);         // both idle unless the flag is set
-            fin(f.ts, f.ntile, f.splits, nullptr, f.redo);
+            direct(f.redo);                                         // idle unless the flag is set
             c->kernels += 2;
             return;
         }
     }
-    int RT = p <= 16 ? 1 : (p <= 32 ? 2 : (p <= 48 ? 3 : 4));
-    const int TS = 16 * RT, ntile = (p + TS - 1) / TS, npair = ntile * (ntile + 1) / 2;
-    int64_t splits = std::max<int64_t>(1, std::min<int64_t>((c->n + 255) / 256, (152LL * 4) / npair + 1));
-    const int64_t rps = ((c->n + splits - 1) / splits + 15) / 16 * 16;
-    splits = (c->n + rps - 1) / rps;
-    direct(TS, ntile, splits, rps, nullptr);
-    fin(TS, ntile, splits);
+    direct(nullptr);
 }
 
 template <> bool pcg_zc<double>(const ofks_ctx *, int) { return false; }

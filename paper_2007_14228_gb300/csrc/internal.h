@@ -386,7 +386,7 @@ constexpr int GRAM_DIG_MIN = 16;
 constexpr float GRAM_DIG_LEAST = 0x1p-100f;
 struct GramDig {
     int ts = 0, ntile = 0;                       // tiles of ts columns, ntile per side
-    int64_t splits = 0, rps = 0;                 // ranges of rps rows
+    int64_t splits = 0;                          // ranges of rows
     float *slack = nullptr;                      // per partial, how far its digits are from too coarse
     int *redo = nullptr;                         // set by k_gram_fin where an entry's are (device)
 };

@@ -96,7 +96,7 @@ def test_every_entry_of_the_gradient(ofks, p, kind):
     assert np.all(np.abs(G - ref) <= 1.001 * bound + 1e-307 * 2.0 ** -40)
 
 
-# Lambda0 = X^T H X and S = X^T B X: sums of 64 rows by digits, or direct sums over at most 128 rows, added over
+# Lambda0 = X^T H X and S = X^T B X: sums of 64 rows by digits, or direct sums over at most 256 rows, added over
 # the ranges of rows
 @pytest.mark.parametrize("kind", ["plain", "spikes", "localized", "graded"])
 @pytest.mark.parametrize("p", [13, 16, 17, 23, 32, 33, 41, 48, 49, 64, 65, 97, 129])
@@ -108,7 +108,7 @@ def test_every_entry_of_the_grams(ofks, p, kind):
     for A, got in ((f["HX"], f["Lambda0"]), (f["BX"], f["S"])):
         ref = np.triu(X.astype(Q).T @ A.astype(Q))
         ref = ref + np.triu(ref, 1).T
-        bound = (128 + len(X) / 64 + 3) * 2.0 ** -53 * np.triu(np.abs(X).T @ np.abs(A))
+        bound = (256 + len(X) / 64 + 3) * 2.0 ** -53 * np.triu(np.abs(X).T @ np.abs(A))
         bound = np.maximum(bound, bound.T)
         assert np.all(np.abs(got - ref) <= 1.001 * bound + 1e-307 * 2.0 ** -40)
 
